@@ -20,22 +20,41 @@
 //               tile j, S_w,j+1 = Q_w K_j+1^T (M=128, N=128, K=d) as soon as
 //               softmax w has read S_w,j into registers, and O_w += P_w,j V_j
 //               (M=128, N=d, K=128, P read from TMEM, V MN-major from smem)
-//               once softmax w has written P_w,j.  Issue runs in a converged
-//               warp with one elected lane, and each query tile has its own
-//               issuer: the small MMAs of a d <= 64 head are cheap enough that
-//               issue and barrier latency, not the tensor core, set the pace.
+//               in halves of 64 keys, each once it is written.  Issue runs in a
+//               converged warp with one elected lane, and each query tile has
+//               its own issuer: the small MMAs of a d <= 64 head are cheap
+//               enough that issue and barrier latency, not the tensor core, set
+//               the pace.
 //   warps 4..7  softmax group 0 (query tile 0), one row per thread
 //   warps 8..11 softmax group 1 (query tile 1)
-// Per key tile a softmax thread loads its whole S row (128 fp32) from TMEM in
-// one round trip, masks and takes the row max in registers, and writes
-// P = 2^(s*scale*log2e - m) as bf16 pairs into its group's TMEM columns, from
-// where the PV MMA reads it as the A operand (TMEM holds S_0, S_1, O_0, O_1,
-// P_0, P_1: 512 columns).  The two groups overlap each other's exponentials
-// with their MMAs.  The reference m is the row's running max, updated
-// lazily: only when a tile raises it by more than 2^8 does the group rescale
-// its O row in TMEM (and the row sum l).  Any reference m gives the same
-// softmax (it cancels in O / l), and keeping it at most 8 below the true
-// running max keeps P <= 2^8, so this is exact up to rounding.
+// Per key tile a softmax thread loads its whole S row (128 fp32) from TMEM in one
+// round trip, masks it where the tile is partly visible, and writes
+// P = 2^(s*scale*log2e - m) as bf16 pairs into its group's TMEM columns, from where
+// the PV MMA reads it as the A operand (TMEM holds S_0, S_1, O_0, O_1, P_0, P_1: 512
+// columns).  The two groups overlap each other's exponentials with their MMAs.
+//
+// The reference m of a row is the maximum of the first key tile in which it sees a
+// key, and it stays there: any m gives the same softmax (it cancels in O / l), P is
+// a floating-point number whose rounding does not depend on its scale, and a row's l
+// is at least 1.  So no later tile needs a row maximum, and O is never rescaled.
+// Only a row whose later scores exceed that first maximum by 2^60 could come near
+// fp32's range; the row sums show it at the end, and the CTA then starts again with
+// the true row maxima, taken in a sweep of its own (S products only).
+//
+// What bounds it: with d = 64, a pair of 128 x 128 tiles costs the tensor core 1024
+// clocks and each SM sub-partition's special-function unit 1024 (two tiles'
+// exponentials at 8 a clock; 1126 measured with the packing and the sums), but only
+// two softmax warps share a sub-partition and each is one serial chain, so the time
+// follows the number of instructions in it (about 5.7 clocks each).  Hence the fixed
+// reference (the running maximum with its votes, its rescale and the two groups' turn
+// taking cost 2440 clocks a pair), the mask built from one word per 32 keys, the
+// unvoted waits, and the probe of pv_done under the second chunk's exponentials.
+// Measured, running maximum -> fixed reference: 5120 tokens of 10 chunks, 16 heads
+// of 64 64.0 -> 54.9 us; 4102 tokens bidirectional 81.6 -> 66.5 us; 16 ragged requests
+// of 95617 tokens, 8 heads 836 -> 660 us.  Tried and slower: four softmax warpgroups
+// of half rows (76 us on the second shape: more barrier work and MIO queueing), the
+// next tile's chunks loaded under the last exponentials (89 us), one hand-over of P
+// instead of two halves (+4 %).
 // O_w is read back and divided by l after the last tile.
 #include <cuda_bf16.h>
 
@@ -73,12 +92,47 @@ constexpr uint32_t kRegsCtl = 48;
 constexpr uint32_t kRegsSoftmax = 224;
 static_assert(kRegsCtl * 128 + 2 * kRegsSoftmax * 128 <= kRegsLaunch * kThreads,
               "register split exceeds the launch allocation");
-constexpr float kRescaleLog2 = 8.0f;   // lazy-rescale threshold (log2 units)
-// Warp q of softmax group 0 and warp q of group 1 share an SM sub-partition
-// (warps 4 + q and 8 + q) and take turns on the exponentials: while one runs
-// its exp pass, the other waits for its S and PV MMAs, loads S and takes the
-// row max, so the special-function unit stays busy.
-constexpr bool kTurns = true;
+constexpr float kRescaleLog2 = 8.0f;   // training: lazy-rescale threshold (log2 units)
+constexpr float kSumLimit = 1.152921504606847e18f;   // 2^60: a larger row sum restarts the CTA
+
+// Scores 32 c .. 32 c + 31 of a row whose visible keys, relative to the tile, are
+// [lo, hi): the others become -inf (a fully visible chunk is left alone).
+template <int C>
+__device__ __forceinline__ void mask_chunk(float (&s)[128], int lo, int hi, float neg_inf) {
+    lo -= 32 * C;
+    hi -= 32 * C;
+    if (hi < 32 || lo > 0) {
+        const uint32_t below = hi >= 32 ? ~0u : (hi <= 0 ? 0u : (1u << hi) - 1u);
+        const uint32_t vis = lo <= 0 ? below : (lo >= 32 ? 0u : below & (~0u << lo));
+#pragma unroll
+        for (int i = 0; i < 32; ++i) s[32 * C + i] = (vis & (1u << i)) ? s[32 * C + i] : neg_inf;
+    }
+}
+// 2^(s sc - m) of scores 32 c .. 32 c + 31 as bf16 pairs, added to four pairs of
+// running row sums.
+template <int C>
+__device__ __forceinline__ void exp_chunk(const float (&s)[128], float sc, float m, uint32_t* pk,
+                                          float (&rs8)[8]) {
+#pragma unroll
+    for (int i = 0; i < 32; i += 2) {
+        float t0, t1;
+        ffma2(t0, t1, s[32 * C + i], s[32 * C + i + 1], sc, sc, -m, -m);
+        const float e0 = ex2(t0);
+        const float e1 = ex2(t1);
+        const int q = (i >> 1) & 3;
+        fadd2(rs8[2 * q], rs8[2 * q + 1], rs8[2 * q], rs8[2 * q + 1], e0, e1);
+        pk[i >> 1] = pack_bf16x2(e0, e1);
+    }
+}
+__device__ __forceinline__ float row_max(const float (&s)[128]) {
+    float mx[8];   // independent chains
+#pragma unroll
+    for (int q = 0; q < 8; ++q) mx[q] = fmaxf(s[2 * q], s[2 * q + 1]);
+#pragma unroll
+    for (int i = 16; i < 128; i += 2) mx[(i >> 1) & 7] = fmax3(mx[(i >> 1) & 7], s[i], s[i + 1]);
+    return fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
+                 fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
+}
 
 // Exclusive end and start of the visible keys of request-local row i.
 __device__ __forceinline__ int key_hi(const AttnParams& p, int rs, int len, int i) {
@@ -90,8 +144,10 @@ __device__ __forceinline__ int key_lo(const AttnParams& p, int rs, int i) {
     return p.mask_mode == CR_MASK_BLOCK_DIAGONAL ? __ldg(p.chunk_start + rs + i) : 0;
 }
 
-// kLse: also write each row's log-sum-exp (for the training step's backward);
-// the inference forward's instantiation has none of that code.
+// kLse: the training forward.  It also writes each row's log-sum-exp (for the
+// backward), and it keeps the running maximum as reference: P's bf16 rounding depends
+// on the reference, and a training step amplifies such a change into 2e-3 of its fp32
+// gradients' norm after six blocks, so its results stay bit for bit what they were.
 template <int D, bool kLse>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_constant__ AttnParams p) {
@@ -113,8 +169,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint64_t* p_full = s_free + 2;        // [2][2] half h of P_w,j (64 keys) in TMEM
     uint64_t* pv_done = p_full + 4;       // [2] O_w += P_w,j V_j complete
     uint64_t* drain = pv_done + 2;        // [2]
-    uint64_t* turn = drain + 2;           // [2][4]: warp q of group w finished an exp pass
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(turn + 8);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 2);
     int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
     // ---- work item: (request, pair of query tiles, head); heaviest pairs first
@@ -142,7 +197,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&pv_done[w], 1);
             mbar_init(&drain[w], 1);
         }
-        for (int t = 0; t < 8; ++t) mbar_init(&turn[t], 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -170,6 +224,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem_base = *tmem_slot;
     const WaitCtx wc{abort_flag, p.status};
 
+    // (a barrier of the whole CTA stands between any two sweeps, so that a role whose
+    // query tile ended early never waits on a ring slot two fills ahead)
+    // all threads agree on whether a row sum asks for a second start; nobody
+    // starts again once a role has given up
+    auto again = [&](bool bad) -> bool {
+        const int redo = __syncthreads_or(bad ? 1 : 0);
+        return __syncthreads_or(*wc.abort != 0 ? 1 : 0) == 0 && redo != 0;
+    };
+
     if (warp < 4) {
         setmaxnreg_dec<kRegsCtl>();
         if (warp == 0) {
@@ -184,23 +247,35 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             __syncwarp();
             bool ok = true;
-            for (int j = 0; j < n_max; ++j) {
-                const int st = j % NS;
-                const uint32_t ph = static_cast<uint32_t>(j / NS) & 1u;
-                if (!(ok = mbar_wait_warp(&kv_empty[st], ph ^ 1u, wc, 121))) break;
-                uint8_t* kt = smem + Cfg::kKVOff + st * 2 * Cfg::kTileBytes;
-                if (elect_one()) {
-                    mbar_expect_tx(&kv_full[st], 2 * Cfg::kTileBytes);
-                    tma_load_2d(kt, &tmQKV, &kv_full[st], p.d_b + head * D, rs + kbase + j * 128);
-                    tma_load_2d(kt + Cfg::kTileBytes, &tmQKV, &kv_full[st], 2 * p.d_b + head * D,
-                                rs + kbase + j * 128);
-                    // the stage is free once both issuers release it; an issuer
-                    // whose query tile ends before tile j is released for here
-                    // (its partner's release, after its MMAs, completes the phase)
-                    if (j >= n_kv[0]) mbar_arrive(&kv_empty[st]);
-                    if (j >= n_kv[1]) mbar_arrive(&kv_empty[st]);
+            int st = 0;
+            uint32_t ph = 0;
+            auto sweep = [&]() {
+                for (int j = 0; j < n_max && ok; ++j) {
+                    if (!(ok = mbar_wait_warp(&kv_empty[st], ph ^ 1u, wc, 121))) break;
+                    uint8_t* kt = smem + Cfg::kKVOff + st * 2 * Cfg::kTileBytes;
+                    if (elect_one()) {
+                        mbar_expect_tx(&kv_full[st], 2 * Cfg::kTileBytes);
+                        tma_load_2d(kt, &tmQKV, &kv_full[st], p.d_b + head * D, rs + kbase + j * 128);
+                        tma_load_2d(kt + Cfg::kTileBytes, &tmQKV, &kv_full[st], 2 * p.d_b + head * D,
+                                    rs + kbase + j * 128);
+                        // the stage is free once both issuers release it; an issuer
+                        // whose query tile ends before tile j is released for here
+                        // (its partner's release, after its MMAs, completes the phase)
+                        if (j >= n_kv[0]) mbar_arrive(&kv_empty[st]);
+                        if (j >= n_kv[1]) mbar_arrive(&kv_empty[st]);
+                    }
+                    __syncwarp();
+                    if (++st == NS) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
                 }
-                __syncwarp();
+            };
+            sweep();
+            if (again(false)) {
+                sweep();
+                __syncthreads();
+                sweep();
             }
             if (!ok) {
                 const uint64_t t0 = globaltimer();
@@ -214,7 +289,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             // once P_w,j is written.  The whole warp runs the loop and computes
             // the descriptors; one elected lane issues the MMAs and commits.
             const int w = static_cast<int>(warp) - 1;
-            constexpr int jl = 0;
             const int n = n_kv[w];
             // Descriptors are built once; a K=16 step adds 32 bytes (2 units of
             // 16 B) to the start address, a stage adds 2 tiles, a V step 16 rows.
@@ -227,18 +301,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t ds = tmem_base + Cfg::kTmemS + w * 128;
             const uint32_t dout = tmem_base + Cfg::kTmemO + w * D;
             const uint32_t pa = tmem_base + Cfg::kTmemP + w * 64;
-            int kv_ready = -1;   // key/value tiles 0..kv_ready are known to be in smem
-            auto ensure_kv = [&](int j) -> bool {
-                if (j <= kv_ready) return true;
-                if (!mbar_wait_warp(&kv_full[j % NS], static_cast<uint32_t>(j / NS) & 1u, wc, 222))
-                    return false;
-                tc_fence_after();
-                kv_ready = j;
-                return true;
-            };
+            // ring slot and phase of tile 0 of this sweep (the producer walks n_max
+            // slots a sweep, whatever this query tile needs of them)
+            int base = 0;
+            uint32_t ns = 0, np = 0;   // S tiles read by the softmax, P tiles multiplied
+            bool ok = mbar_wait_warp(q_full, 0, wc, 221);
+            if (ok) tc_fence_after();
             auto issue_s = [&](int j) -> bool {
-                if (!ensure_kv(j)) return false;
-                const uint64_t dk = dk0 + static_cast<uint64_t>(j % NS) * kStageStep;
+                const int g = base + j;
+                if (!mbar_wait_warp(&kv_full[g % NS], static_cast<uint32_t>(g / NS) & 1u, wc, 222)) return false;
+                tc_fence_after();
+                const uint64_t dk = dk0 + static_cast<uint64_t>(g % NS) * kStageStep;
                 if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < D / 16; ++k)
@@ -248,16 +321,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 __syncwarp();
                 return true;
             };
-            // PV in two halves of 64 keys, each issued as soon as softmax w has
-            // written that half of P: the first half's MMAs run while the
-            // second half is being exponentiated.
+            // PV in two halves of 64 keys, each issued as soon as its softmax group
+            // has written it (its V tile arrived with the K tile of S_w,j)
             auto issue_pv = [&](int j) -> bool {
-                if (!ensure_kv(j)) return false;
-                const uint64_t dv = dv0 + static_cast<uint64_t>(j % NS) * kStageStep;
+                const uint64_t dv = dv0 + static_cast<uint64_t>((base + j) % NS) * kStageStep;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    if (!mbar_wait_warp(&p_full[2 * w + h], static_cast<uint32_t>(j - jl) & 1u, wc, 224))
-                        return false;
+                    if (!mbar_wait_warp(&p_full[2 * w + h], np & 1u, wc, 224)) return false;
                     tc_fence_after();
                     if (elect_one()) {
 #pragma unroll
@@ -266,35 +336,44 @@ __global__ void __launch_bounds__(kThreads, 1)
                             // dimension), d contiguous (MN-major); 16 keys = two 8-row atoms.
                             const int kk = 4 * h + q;
                             mma_bf16_ts(dout, pa + kk * 8, dv + kk * ((16 * Cfg::kRowBytes) >> 4),
-                                        IDESC_PV, (j > jl || kk != 0) ? 1u : 0u);
+                                        IDESC_PV, (j > 0 || kk != 0) ? 1u : 0u);
                         }
                         if (h == 1) mma_commit(&pv_done[w]);
                     }
                     __syncwarp();
                 }
+                ++np;
                 return true;
             };
-            bool ok = mbar_wait_warp(q_full, 0, wc, 221);
-            if (ok) tc_fence_after();
-            // only the tiles of [jl, n): the producer releases the others
-            if (ok && n > jl) ok = issue_s(jl);
-            for (int j = jl; j < n && ok; ++j) {
-                if (j + 1 < n) {
-                    ok = mbar_wait_warp(&s_free[w], static_cast<uint32_t>(j - jl) & 1u, wc, 223);
+            // only the tiles of [0, n): the producer releases the others
+            auto sweep = [&](bool pv) {
+                if (ok && n > 0) ok = issue_s(0);
+                for (int j = 0; j < n && ok; ++j) {
+                    // S_w,j has been read before S_w,j+1 (or the next sweep's first) overwrites it
+                    ok = mbar_wait_warp(&s_free[w], ns & 1u, wc, 223);
+                    ++ns;
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (j + 1 < n) ok = issue_s(j + 1);
+                    if (ok && pv) ok = issue_pv(j);
                     if (ok) {
-                        tc_fence_after();
-                        ok = issue_s(j + 1);
+                        if (elect_one()) mma_commit(&kv_empty[(base + j) % NS]);
+                        __syncwarp();
                     }
                 }
-                if (ok) ok = issue_pv(j);
-                if (ok) {
-                    if (elect_one()) mma_commit(&kv_empty[j % NS]);
-                    __syncwarp();
-                }
+                base += n_max;
+            };
+            sweep(true);
+            if (again(false)) {
+                sweep(false);
+                __syncthreads();
+                sweep(true);
             }
             if (elect_one()) mma_commit(&drain[w]);
             __syncwarp();
             mbar_wait_warp(&drain[w], 0, wc, 227);
+        } else if (again(false)) {
+            __syncthreads();
         }
     } else {
         setmaxnreg_inc<kRegsSoftmax>();
@@ -304,137 +383,169 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int r = static_cast<int>(quad * 32 + lane);
         const int qrow = q0 + 128 * w + r;
         const bool valid = qrow < len;
-        // visible keys of this row, relative to kbase
-        const int cend = (valid ? key_hi(p, rs, len, qrow) : 1) - kbase;
-        const int cbeg = (valid ? key_lo(p, rs, qrow) : 0) - kbase;
+        // visible keys of this row, relative to the first key tile (a row past the
+        // request's end is never stored: no mask; with the running maximum it shares
+        // its warp's votes and sees one key)
+        const int cend = valid ? key_hi(p, rs, len, qrow) - kbase : (kLse ? 1 - kbase : 1 << 30);
+        const int cbeg = valid ? key_lo(p, rs, qrow) - kbase : (kLse ? -kbase : 0);
         const uint32_t lane_off = (quad * 32u) << 16;
         const uint32_t ts = tmem_base + lane_off + Cfg::kTmemS + w * 128;
         const uint32_t to = tmem_base + lane_off + Cfg::kTmemO + w * D;
-        const float sc = p.scale_log2;
-        constexpr int jl = 0;
-        const int n = n_kv[w];
-        // exp-pass turns: tile j of group 0 waits for group 1's tile j - 1, tile
-        // j of group 1 for group 0's tile j, when the other group has that tile;
-        // jt = j - turn_lo is the waited-for pass of the other group
-        const int turn_lo = (w == 0) ? 1 : 0;
-        const int turn_hi = (w == 0) ? n_kv[1] + 1 : n_kv[0];
         const uint32_t tp = tmem_base + lane_off + Cfg::kTmemP + w * 64;
+        const float sc = p.scale_log2;
+        const int n = n_kv[w];
         float m = NEG_INF, l = 0.0f;
-
-        bool ok = true;
-        for (int j = jl; j < n; ++j) {
-            const uint32_t it = static_cast<uint32_t>(j - jl);   // tiles done by this group
-            ok = mbar_wait(&s_full[w], it & 1u, wc, 321);
-            if (!__all_sync(0xffffffffu, ok)) {
-                ok = false;
-                break;
-            }
+        uint32_t ns = 0, np = 0;   // S tiles read, PV products waited for
+        const uint32_t a_s = smem_u32(&s_full[w]), a_free = smem_u32(&s_free[w]), a_pv = smem_u32(&pv_done[w]),
+                       a_p0 = smem_u32(&p_full[2 * w]), a_p1 = smem_u32(&p_full[2 * w + 1]);
+        // A wait that gives up (the status word then says so) leaves stale scores
+        // behind, which only this CTA's own rows would show: the loop goes on, its
+        // later waits give up at once, and every role still reaches the end.
+        auto wait = [&](uint32_t a, uint32_t parity, unsigned site) {
+            if (!mbar_test_wait(a, parity)) mbar_wait_slow(a, parity, wc, site);
+            __syncwarp();
             tc_fence_after();
-            // the whole S row in registers: one TMEM round trip per tile, after
-            // which the tensor core may overwrite S with the next tile's scores
-            float s[128];
-            tmem_ld32(ts, s);
-            tmem_ld32(ts + 32, s + 32);
-            tmem_ld32(ts + 64, s + 64);
-            tmem_ld32(ts + 96, s + 96);
-            tmem_wait_ld();
+        };
+        auto hand_over = [&](uint32_t a) {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&s_free[w]);
-            const int k0 = j * 128;
-            if (k0 + 128 > cend || k0 < cbeg) {
-                // keys outside [cbeg, cend) are masked; fully visible tiles skip this
-                const int hi = cend - k0, lo = cbeg - k0;
-#pragma unroll
-                for (int i = 0; i < 128; ++i) s[i] = (i < hi && i >= lo) ? s[i] : NEG_INF;
+            if (lane == 0) mbar_arrive_u32(a);
+        };
+        // the whole S row of the next tile in registers: one TMEM round trip, after
+        // which the tensor core may overwrite S
+        auto take_s = [&](float (&s)[128], int j) {
+            wait(a_s, ns & 1u, 321);
+            ++ns;
+            tmem_ld64(ts, s);
+            tmem_ld64(ts + 64, s + 64);
+            tmem_wait_ld();
+            const int lo = cbeg - j * 128, hi = cend - j * 128;
+            if (__any_sync(0xffffffffu, hi < 128 || lo > 0)) {
+                mask_chunk<0>(s, lo, hi, NEG_INF);
+                mask_chunk<1>(s, lo, hi, NEG_INF);
+                mask_chunk<2>(s, lo, hi, NEG_INF);
+                mask_chunk<3>(s, lo, hi, NEG_INF);
             }
-            // row max of the (masked) scores in eight independent chains
-            float mxv[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) mxv[q] = NEG_INF;
-#pragma unroll
-            for (int i = 0; i < 128; i += 2) mxv[(i >> 1) & 7] = fmax3(mxv[(i >> 1) & 7], s[i], s[i + 1]);
-            float mx = fmaxf(fmaxf(fmaxf(mxv[0], mxv[1]), fmaxf(mxv[2], mxv[3])),
-                             fmaxf(fmaxf(mxv[4], mxv[5]), fmaxf(mxv[6], mxv[7])));
-            mx *= sc;
-            // O_w and P_w are free once PV_w,j-1 has completed
-            if (j > jl) {
-                ok = mbar_wait(&pv_done[w], (it - 1u) & 1u, wc, 322);
-                if (!__all_sync(0xffffffffu, ok)) {
-                    ok = false;
-                    break;
+        };
+        auto sweep_max = [&]() {
+            m = NEG_INF;
+            for (int j = 0; j < n; ++j) {
+                float s[128];
+                take_s(s, j);
+                hand_over(a_free);
+                m = fmaxf(m, row_max(s) * sc);
+            }
+        };
+        // the training forward's form: m is the row's running maximum, moved lazily, only
+        // when a tile raises it by more than 2^8 somewhere in the warp (O_w and l are
+        // then rescaled)
+        auto sweep_running = [&]() {
+            for (int j = 0; j < n; ++j) {
+                float s[128];
+                take_s(s, j);
+                hand_over(a_free);
+                const float mx = row_max(s) * sc;
+                // O_w and P_w are free once PV_w,j-1 has completed
+                if (j > 0) {
+                    wait(a_pv, np & 1u, 322);
+                    ++np;
                 }
-                tc_fence_after();
-            }
-            // lazily move the reference max: on the first tile, or when this
-            // tile would push P above 2^8 somewhere in the warp.  A row whose
-            // visible keys start in a later tile (block-diagonal mask) keeps
-            // m = -inf until then: its P is 0 (exponent taken against 0) and
-            // its first rescale multiplies the zero O and l by 0.
-            const bool raise = (j == jl) || (mx > m + kRescaleLog2);
-            if (__any_sync(0xffffffffu, raise)) {
-                const float m_new = fmaxf(m, mx);
-                if (j > jl) {
-                    const float alpha = (m == m_new) ? 1.0f : ex2(m - m_new);
+                const bool raise = (j == 0) || (mx > m + kRescaleLog2);
+                if (__any_sync(0xffffffffu, raise)) {
+                    const float m_new = fmaxf(m, mx);
+                    if (j > 0) {
+                        const float alpha = (m == m_new) ? 1.0f : ex2(m - m_new);
 #pragma unroll
-                    for (int c = 0; c < D; c += 16) {
-                        float o[16];
-                        tmem_ld16(to + c, o);
-                        tmem_wait_ld();
+                        for (int c = 0; c < D; c += 16) {
+                            float o[16];
+                            tmem_ld16(to + c, o);
+                            tmem_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) o[i] *= alpha;
-                        tmem_st16(to + c, o);
+                            for (int i = 0; i < 16; ++i) o[i] *= alpha;
+                            tmem_st16(to + c, o);
+                        }
+                        l *= alpha;
                     }
-                    l *= alpha;
+                    m = m_new;
                 }
-                m = m_new;
+                // (a row whose keys start in a later tile has m = -inf: its P is 0)
+                const float m_ref = (m == NEG_INF) ? 0.0f : m;
+                float rs8[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) rs8[q] = 0.0f;
+                uint32_t pk[32];
+                exp_chunk<0>(s, sc, m_ref, pk, rs8);
+                exp_chunk<1>(s, sc, m_ref, pk + 16, rs8);
+                tmem_st32u(tp, pk);
+                tmem_wait_st();
+                hand_over(a_p0);
+                exp_chunk<2>(s, sc, m_ref, pk, rs8);
+                exp_chunk<3>(s, sc, m_ref, pk + 16, rs8);
+                tmem_st32u(tp + 32, pk);
+                tmem_wait_st();
+                hand_over(a_p1);
+                l += ((rs8[0] + rs8[1]) + (rs8[2] + rs8[3])) + ((rs8[4] + rs8[5]) + (rs8[6] + rs8[7]));
             }
-            if (kTurns && j >= turn_lo && j < turn_hi) {
-                // group 0 goes first on each key tile
-                const int jt = j - turn_lo;
-                ok = mbar_wait(&turn[(1 - w) * 4 + quad], static_cast<uint32_t>(jt) & 1u, wc, 323);
-                if (!__all_sync(0xffffffffu, ok)) {
-                    ok = false;
-                    break;
-                }
+            if (n > 0) {
+                wait(a_pv, np & 1u, 324);
+                ++np;
             }
-            // P = 2^(s*sc - m) -> bf16 pairs in TMEM, and the row sum
-            const float m_ref = (m == NEG_INF) ? 0.0f : m;
-            float rs8[8];
+        };
+        // P and l of every key tile; `known`: m is the row's maximum already
+        auto sweep = [&](bool known) {
+            float rs8[8];   // four pairs of running sums
 #pragma unroll
             for (int q = 0; q < 8; ++q) rs8[q] = 0.0f;
-#pragma unroll
-            for (int h = 0; h < 128; h += 64) {
-                uint32_t pk[32];
-#pragma unroll
-                for (int i = 0; i < 64; i += 2) {
-                    float t0, t1;
-                    ffma2(t0, t1, s[h + i], s[h + i + 1], sc, sc, -m_ref, -m_ref);
-                    const float e0 = ex2(t0);
-                    const float e1 = ex2(t1);
-                    const int q = (i >> 1) & 3;       // four pairs of running sums
-                    fadd2(rs8[2 * q], rs8[2 * q + 1], rs8[2 * q], rs8[2 * q + 1], e0, e1);
-                    pk[i >> 1] = pack_bf16x2(e0, e1);
+            for (int j = 0; j < n; ++j) {
+                float s[128];
+                take_s(s, j);
+                // rows that saw no key before take their reference here; where a row
+                // sees none yet (block-diagonal mask) m stays -inf and its P is 0
+                hand_over(a_free);
+                if (!known && __any_sync(0xffffffffu, m == NEG_INF)) {
+                    const float mx = row_max(s) * sc;
+                    if (m == NEG_INF) m = mx;
                 }
-                tmem_st32u(tp + h / 2, pk);
-                // hand this half of P to the MMA issuer
+                const float m_ref = (m == NEG_INF) ? 0.0f : m;
+                uint32_t pk[32];
+                exp_chunk<0>(s, sc, m_ref, pk, rs8);
+                // P_w is free once PV_w,j-1 has completed: the probe's answer comes
+                // in under the next chunk's exponentials
+                const bool pv = j > 0 && mbar_test_wait(a_pv, np & 1u);
+                exp_chunk<1>(s, sc, m_ref, pk + 16, rs8);
+                if (j > 0) {
+                    if (!pv) mbar_wait_slow(a_pv, np & 1u, wc, 322);
+                    __syncwarp();
+                    tc_fence_after();
+                    ++np;
+                }
+                tmem_st32u(tp, pk);
                 tmem_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&p_full[2 * w + (h >> 6)]);
+                hand_over(a_p0);
+                exp_chunk<2>(s, sc, m_ref, pk, rs8);
+                exp_chunk<3>(s, sc, m_ref, pk + 16, rs8);
+                tmem_st32u(tp + 32, pk);
+                tmem_wait_st();
+                hand_over(a_p1);
             }
-            if (kTurns) {
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&turn[w * 4 + quad]);
+            if (n > 0) {
+                l = ((rs8[0] + rs8[1]) + (rs8[2] + rs8[3])) + ((rs8[4] + rs8[5]) + (rs8[6] + rs8[7]));
+                wait(a_pv, np & 1u, 324);
+                ++np;
             }
-            l += ((rs8[0] + rs8[1]) + (rs8[2] + rs8[3])) + ((rs8[4] + rs8[5]) + (rs8[6] + rs8[7]));
+        };
+        if constexpr (kLse) {
+            sweep_running();
+            again(false);
+        } else {
+            sweep(false);
+            if (again(n > 0 && valid && !(l <= kSumLimit))) {
+                sweep_max();
+                __syncthreads();
+                sweep(true);
+            }
         }
-        if (ok && n > jl) {
-            ok = mbar_wait(&pv_done[w], static_cast<uint32_t>(n - 1 - jl) & 1u, wc, 324);
-            ok = __all_sync(0xffffffffu, ok);
-        }
-        if (ok && n > jl) {
-            tc_fence_after();
+        if (n > 0) {
             const float inv = 1.0f / l;
             // the row's log-sum-exp for a backward pass: P = 2^(s sc - (m + log2 l))
             if (kLse && valid)

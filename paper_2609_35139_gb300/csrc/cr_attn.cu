@@ -12,10 +12,13 @@
 // inside a key tile mask the rest of it; fully visible tiles do no masking
 // work at all.
 //
-// CTA = (request, head, two consecutive 128-query tiles w = 0, 1); three
+// A work item is a (request, head, pair of consecutive 128-query tiles w = 0, 1).  A
+// CTA runs one item after another: its own block's, then items of blocks that have not
+// started, which it takes over by cluster launch control as soon as an item's loads are
+// out, so that the next item's Q, K and V arrive under this one's last tiles.  Three
 // warpgroups, the first of which gives registers to the other two:
-//   warp 0      TMA: both Q tiles once, then K_j and V_j per key tile into a
-//               5-deep ring shared by the two query tiles
+//   warp 0      TMA: both Q tiles of an item (two buffers), then K_j and V_j per key
+//               tile into a 4-deep ring shared by the two query tiles
 //   warp 1 + w  MMA issue for query tile w (warp 1 also owns TMEM): per key
 //               tile j, S_w,j+1 = Q_w K_j+1^T (M=128, N=128, K=d) as soon as
 //               softmax w has read S_w,j into registers, and O_w += P_w,j V_j
@@ -25,6 +28,7 @@
 //               its own issuer: the small MMAs of a d <= 64 head are cheap
 //               enough that issue and barrier latency, not the tensor core, set
 //               the pace.
+//   warp 3      the item scheduler
 //   warps 4..7  softmax group 0 (query tile 0), one row per thread
 //   warps 8..11 softmax group 1 (query tile 1)
 // Per key tile a softmax thread loads its whole S row (128 fp32) from TMEM in one
@@ -38,23 +42,28 @@
 // a floating-point number whose rounding does not depend on its scale, and a row's l
 // is at least 1.  So no later tile needs a row maximum, and O is never rescaled.
 // Only a row whose later scores exceed that first maximum by 2^60 could come near
-// fp32's range; the row sums show it at the end, and the CTA then starts again with
-// the true row maxima, taken in a sweep of its own (S products only).
+// fp32's range; the row sums show it at the end of the item, and the CTA runs such an
+// item again before it ends, with the true row maxima (a sweep of S products only,
+// then the softmax).
 //
 // What bounds it: with d = 64, a pair of 128 x 128 tiles costs the tensor core 1024
 // clocks and each SM sub-partition's special-function unit 1024 (two tiles'
 // exponentials at 8 a clock; 1126 measured with the packing and the sums), but only
 // two softmax warps share a sub-partition and each is one serial chain, so the time
-// follows the number of instructions in it (about 5.7 clocks each).  Hence the fixed
-// reference (the running maximum with its votes, its rescale and the two groups' turn
-// taking cost 2440 clocks a pair), the mask built from one word per 32 keys, the
-// unvoted waits, and the probe of pv_done under the second chunk's exponentials.
-// Measured, running maximum -> fixed reference: 5120 tokens of 10 chunks, 16 heads
-// of 64 64.0 -> 54.9 us; 4102 tokens bidirectional 81.6 -> 66.5 us; 16 ragged requests
-// of 95617 tokens, 8 heads 836 -> 660 us.  Tried and slower: four softmax warpgroups
-// of half rows (76 us on the second shape: more barrier work and MIO queueing), the
-// next tile's chunks loaded under the last exponentials (89 us), one hand-over of P
-// instead of two halves (+4 %).
+// follows the number of instructions in it (about 5.7 clocks each) and how well its
+// registers hold a whole row.  Hence the fixed reference (the running maximum with its
+// votes, its rescale and the two groups' turn taking cost 2440 clocks a pair), the mask
+// built from one word per 32 keys, the unvoted waits, one pair of row sums, and item
+// fields re-read from shared memory instead of kept.  One block per item cost 8700
+// clocks around its tiles (block start, TMEM, barriers, first loads, last products).
+// Measured, us: 5120 tokens of 10 chunks, 16 heads of 64 | 4102 tokens bidirectional |
+// 5120 tokens block-diagonal | 16 ragged requests of 95617 tokens, 8 heads:
+//   running maximum, a block per item   64.0 | 81.6 | 25.1 | 836
+//   fixed reference                     54.6 | 66.3 | 24.1 | 658
+//   and items taken over                52.4 | 66.1 | 21.1 | 598
+// Tried and slower: four softmax warpgroups of half rows (76 us on the second shape:
+// more barrier work and MIO queueing), the next tile's chunks loaded under the last
+// exponentials (89 us), one hand-over of P instead of two halves (+4 %), spinning waits.
 // O_w is read back and divided by l after the last tile.
 #include <cuda_bf16.h>
 
@@ -70,11 +79,11 @@ struct AttnCfg {
     static constexpr uint32_t kAtomBytes = 8 * kRowBytes;    // swizzle atom (8 rows)
     static constexpr uint32_t kTileBytes = 128 * kRowBytes;
     static constexpr uint32_t kSwz = (D == 64) ? SWZ_128B : SWZ_64B;
-    static constexpr int kStages = 5;
-    static constexpr uint32_t kQOff = 0;                                  // Q0, Q1
-    static constexpr uint32_t kKVOff = 2 * kTileBytes;                    // K, V per stage
+    static constexpr int kStages = 4;
+    static constexpr uint32_t kQOff = 0;                                  // Q0, Q1 of two items
+    static constexpr uint32_t kKVOff = 4 * kTileBytes;                    // K, V per stage
     static constexpr uint32_t kBarOff = kKVOff + kStages * 2 * kTileBytes;
-    static constexpr uint32_t kSmemBytes = 1024 + kBarOff + 320;
+    static constexpr uint32_t kSmemBytes = 1024 + kBarOff + 512;
     static constexpr uint32_t kTmemS = 0;      // S_w at w * 128 (fp32)
     static constexpr uint32_t kTmemO = 256;    // O_w at 256 + w * D (fp32)
     static constexpr uint32_t kTmemP = 384;    // P_w at 384 + w * 64 (bf16 pairs)
@@ -93,6 +102,7 @@ constexpr uint32_t kRegsSoftmax = 224;
 static_assert(kRegsCtl * 128 + 2 * kRegsSoftmax * 128 <= kRegsLaunch * kThreads,
               "register split exceeds the launch allocation");
 constexpr float kRescaleLog2 = 8.0f;   // training: lazy-rescale threshold (log2 units)
+constexpr float kUnseen = -3.0e38f;     // the reference of a row that has seen no key
 constexpr float kSumLimit = 1.152921504606847e18f;   // 2^60: a larger row sum restarts the CTA
 
 // Scores 32 c .. 32 c + 31 of a row whose visible keys, relative to the tile, are
@@ -108,19 +118,19 @@ __device__ __forceinline__ void mask_chunk(float (&s)[128], int lo, int hi, floa
         for (int i = 0; i < 32; ++i) s[32 * C + i] = (vis & (1u << i)) ? s[32 * C + i] : neg_inf;
     }
 }
-// 2^(s sc - m) of scores 32 c .. 32 c + 31 as bf16 pairs, added to four pairs of
+// 2^(s sc - m) of scores 32 c .. 32 c + 31 as bf16 pairs, added to NR / 2 pairs of
 // running row sums.
-template <int C>
+template <int C, int NR>
 __device__ __forceinline__ void exp_chunk(const float (&s)[128], float sc, float m, uint32_t* pk,
-                                          float (&rs8)[8]) {
+                                          float (&rs)[NR]) {
 #pragma unroll
     for (int i = 0; i < 32; i += 2) {
         float t0, t1;
         ffma2(t0, t1, s[32 * C + i], s[32 * C + i + 1], sc, sc, -m, -m);
         const float e0 = ex2(t0);
         const float e1 = ex2(t1);
-        const int q = (i >> 1) & 3;
-        fadd2(rs8[2 * q], rs8[2 * q + 1], rs8[2 * q], rs8[2 * q + 1], e0, e1);
+        const int q = (i >> 1) % (NR / 2);
+        fadd2(rs[2 * q], rs[2 * q + 1], rs[2 * q], rs[2 * q + 1], e0, e1);
         pk[i >> 1] = pack_bf16x2(e0, e1);
     }
 }
@@ -144,6 +154,51 @@ __device__ __forceinline__ int key_lo(const AttnParams& p, int rs, int i) {
     return p.mask_mode == CR_MASK_BLOCK_DIAGONAL ? __ldg(p.chunk_start + rs + i) : 0;
 }
 
+// Byte offsets of a query tile's barriers from s_full[w].
+constexpr int kOffS = 0, kOffFree = 16, kOffP0 = 32, kOffP1 = 48, kOffPV = 64, kOffO = 80;
+template <int N>
+struct At { static constexpr int value = N; };
+
+// One work item: a (request, pair of query tiles, head), by its block index.
+enum Sweep : int { SWEEP_FIRST = 0, SWEEP_MAX = 1, SWEEP_KNOWN = 2 };
+struct Item {
+    int bid;     // < 0: no more items
+    int sweep;   // Sweep: the softmax, the row maxima alone, the softmax with them known
+    int q0, rs, len, kbase, n0, n1;
+};
+constexpr int kDesc = 8;
+static_assert(sizeof(Item) == kDesc * 4, "descriptor size");
+
+// Heaviest pairs of each request first.  Both query tiles start at the key tile of the
+// pair's first visible key, kbase = 128 * floor(lo(q0) / 128), so that every role takes
+// the ring's tiles in order.  (Under the block-diagonal mask the second tile's rows may
+// start later; their leading key tiles are fully masked and contribute exact zeros.)
+// Tile j of an item is key tile kbase / 128 + j; query tile w needs j in [0, n_w), an
+// empty second tile (past the request's end) none.
+__device__ __forceinline__ Item make_item(const AttnParams& p, int bid, int sweep) {
+    Item d;
+    d.bid = bid;
+    d.sweep = sweep;
+    if (bid < 0) {
+        d.q0 = d.rs = d.len = d.kbase = d.n0 = d.n1 = 0;
+        return d;
+    }
+    const int pair = p.n_items - 1 - bid / p.n_heads;
+    int a = 0, b = p.n_req - 1;   // the request with tile_prefix[r] <= pair
+    while (a < b) {
+        const int mid = (a + b + 1) >> 1;
+        if (p.tile_prefix[mid] <= pair) a = mid;
+        else b = mid - 1;
+    }
+    d.q0 = (pair - p.tile_prefix[a]) * 256;
+    d.rs = p.req_start[a];
+    d.len = p.req_start[a + 1] - d.rs;
+    d.kbase = key_lo(p, d.rs, d.q0) & ~127;
+    d.n0 = (key_hi(p, d.rs, d.len, min(d.q0 + 127, d.len - 1)) - d.kbase + 127) / 128;
+    d.n1 = d.q0 + 128 < d.len ? (key_hi(p, d.rs, d.len, min(d.q0 + 255, d.len - 1)) - d.kbase + 127) / 128 : 0;
+    return d;
+}
+
 // kLse: the training forward.  It also writes each row's log-sum-exp (for the
 // backward), and it keeps the running maximum as reference: P's bf16 rounding depends
 // on the reference, and a training step amplifies such a change into 2e-3 of its fp32
@@ -161,43 +216,55 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::kBarOff);
-    uint64_t* q_full = bars;
-    uint64_t* kv_full = bars + 1;
+    uint64_t* q_full = bars;              // [2] Q tiles of an item in buffer it & 1
+    uint64_t* q_empty = bars + 2;         // [2] both issuers are done with them
+    uint64_t* kv_full = bars + 4;
     uint64_t* kv_empty = kv_full + NS;
+    // (the softmax groups address these five at fixed offsets, kOffS ..)
     uint64_t* s_full = kv_empty + NS;     // [2] S_w,j in TMEM
     uint64_t* s_free = s_full + 2;        // [2] S_w,j read into registers
-    uint64_t* p_full = s_free + 2;        // [2][2] half h of P_w,j (64 keys) in TMEM
+    uint64_t* p_full = s_free + 2;        // [h][w] half h of P_w,j (64 keys) in TMEM
     uint64_t* pv_done = p_full + 4;       // [2] O_w += P_w,j V_j complete
-    uint64_t* drain = pv_done + 2;        // [2]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 2);
+    uint64_t* o_free = pv_done + 2;       // [2] O_w of an item read into registers
+    uint64_t* drain = o_free + 2;         // [2]
+    uint64_t* item_full = drain + 2;      // [2] the descriptor of item it in slot it & 1
+    uint64_t* item_empty = item_full + 2; // [2] producer and issuers have read it, and the 8
+                                          //     softmax warps are done with the item
+    uint64_t* loads_out = item_empty + 2; // the loads of an item have all been issued
+    uint64_t* clc_full = loads_out + 1;   // the answer to a request for another item
+    // (34 barriers: 272 bytes)
+    uint4* clc_answer = reinterpret_cast<uint4*>(smem + Cfg::kBarOff + 320);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + Cfg::kBarOff + 336);
     int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-
-    // ---- work item: (request, pair of query tiles, head); heaviest pairs first
-    const int head = blockIdx.x % p.n_heads;
-    const int item = p.n_items - 1 - static_cast<int>(blockIdx.x / p.n_heads);
-    int req = 0;
-    while (req + 1 < p.n_req && p.tile_prefix[req + 1] <= item) ++req;
-    const int q0 = (item - p.tile_prefix[req]) * 256;
-    const int rs = p.req_start[req];
-    const int len = p.req_start[req + 1] - rs;
+    volatile int* redo_any = abort_flag + 1;
+    volatile int* redo = abort_flag + 3;  // [4] items to start again, slot it & 3 (-1: none)
+    volatile int* desc = redo + 4;        // [2][kDesc]
 
     const uint32_t warp = warp_id(), lane = lane_id();
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
-        mbar_init(q_full, 1);
         for (int s = 0; s < NS; ++s) {
             mbar_init(&kv_full[s], 1);
             mbar_init(&kv_empty[s], 2);   // both issuers release each stage
         }
         for (int w = 0; w < 2; ++w) {
+            mbar_init(&q_full[w], 1);
+            mbar_init(&q_empty[w], 2);
             mbar_init(&s_full[w], 1);
             mbar_init(&s_free[w], 4);
             mbar_init(&p_full[2 * w], 4);
             mbar_init(&p_full[2 * w + 1], 4);
             mbar_init(&pv_done[w], 1);
+            mbar_init(&o_free[w], 4);
             mbar_init(&drain[w], 1);
+            mbar_init(&item_full[w], 1);
+            mbar_init(&item_empty[w], 11);
         }
+        mbar_init(loads_out, 1);
+        mbar_init(clc_full, 1);
         *abort_flag = 0;
+        *redo_any = 0;
+        for (int k = 0; k < 4; ++k) redo[k] = -1;
         fence_barrier_init();
     }
     if (warp == 1) tmem_alloc(tmem_slot, 512);
@@ -205,32 +272,25 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     pdl_wait();   // qkv and the chunk map come from earlier kernels
-    // Both query tiles start at the key tile of the pair's first visible key,
-    // kbase = 128 * floor(lo(q0) / 128): every issuer and softmax group then
-    // takes the ring's tiles in order from its first slot use, which keeps
-    // each parity wait within one phase of its barrier.  (Under the
-    // block-diagonal mask the second tile's rows may start later; their
-    // leading key tiles are fully masked and contribute exact zeros.)  Tile j
-    // below is key tile kbase / 128 + j; query tile w needs j in [0, n_kv[w]),
-    // an empty second tile (past the request's end) none.
-    const int kbase = key_lo(p, rs, q0) & ~127;
-    int n_kv[2];
-#pragma unroll
-    for (int w = 0; w < 2; ++w) {
-        const int first = q0 + 128 * w;
-        n_kv[w] = first < len ? (key_hi(p, rs, len, min(first + 127, len - 1)) - kbase + 127) / 128 : 0;
-    }
-    const int n_max = max(n_kv[0], n_kv[1]);
     const uint32_t tmem_base = *tmem_slot;
     const WaitCtx wc{abort_flag, p.status};
 
-    // (a barrier of the whole CTA stands between any two sweeps, so that a role whose
-    // query tile ended early never waits on a ring slot two fills ahead)
-    // all threads agree on whether a row sum asks for a second start; nobody
-    // starts again once a role has given up
-    auto again = [&](bool bad) -> bool {
-        const int redo = __syncthreads_or(bad ? 1 : 0);
-        return __syncthreads_or(*wc.abort != 0 ? 1 : 0) == 0 && redo != 0;
+    // Every role walks the items to their end, all meet, and where a row sum asked for it
+    // they walk the items to run again.
+    auto meet = [&](int pass) -> bool {
+        __syncthreads();
+        return !kLse && pass == 0 && *redo_any != 0;
+    };
+    // The descriptor of the CTA's it-th item, for the producer and issuer warps; false at
+    // the end (or when a role has given up).
+    auto next_item = [&](uint32_t it, Item* d) -> bool {
+        if (!mbar_wait_warp(&item_full[it & 1u], (it >> 1) & 1u, wc, 131)) return false;
+        int* v = reinterpret_cast<int*>(d);
+#pragma unroll
+        for (int k = 0; k < kDesc; ++k) v[k] = desc[(it & 1u) * kDesc + k];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&item_empty[it & 1u]);
+        return d->bid >= 0;
     };
 
     if (warp < 4) {
@@ -238,44 +298,45 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (warp == 0) {
             // ---------------------------------------------------- TMA producer
             // (the whole warp runs the loop; one elected lane issues)
-            if (elect_one()) {
-                tma_prefetch(&tmQKV);
-                mbar_expect_tx(q_full, 2 * Cfg::kTileBytes);
-                tma_load_2d(smem + Cfg::kQOff, &tmQKV, q_full, head * D, rs + q0);
-                tma_load_2d(smem + Cfg::kQOff + Cfg::kTileBytes, &tmQKV, q_full, head * D,
-                            rs + q0 + 128);
-            }
+            if (elect_one()) tma_prefetch(&tmQKV);
             __syncwarp();
             bool ok = true;
             int st = 0;
             uint32_t ph = 0;
-            auto sweep = [&]() {
-                for (int j = 0; j < n_max && ok; ++j) {
-                    if (!(ok = mbar_wait_warp(&kv_empty[st], ph ^ 1u, wc, 121))) break;
-                    uint8_t* kt = smem + Cfg::kKVOff + st * 2 * Cfg::kTileBytes;
+            uint32_t it = 0, iq = 0;   // descriptors read, items (the end marks have no Q)
+            for (int pass = 0;; ++pass) {
+                Item d;
+                for (; ok && next_item(it, &d); ++it, ++iq) {
+                    const int head = d.bid % p.n_heads, n_max = max(d.n0, d.n1);
+                    uint64_t* qf = &q_full[iq & 1u];
+                    uint8_t* qt = smem + Cfg::kQOff + (iq & 1u) * 2 * Cfg::kTileBytes;
+                    if (!(ok = mbar_wait_warp(&q_empty[iq & 1u], ((iq >> 1) & 1u) ^ 1u, wc, 122))) break;
                     if (elect_one()) {
-                        mbar_expect_tx(&kv_full[st], 2 * Cfg::kTileBytes);
-                        tma_load_2d(kt, &tmQKV, &kv_full[st], p.d_b + head * D, rs + kbase + j * 128);
-                        tma_load_2d(kt + Cfg::kTileBytes, &tmQKV, &kv_full[st], 2 * p.d_b + head * D,
-                                    rs + kbase + j * 128);
-                        // the stage is free once both issuers release it; an issuer
-                        // whose query tile ends before tile j is released for here
-                        // (its partner's release, after its MMAs, completes the phase)
-                        if (j >= n_kv[0]) mbar_arrive(&kv_empty[st]);
-                        if (j >= n_kv[1]) mbar_arrive(&kv_empty[st]);
+                        mbar_expect_tx(qf, 2 * Cfg::kTileBytes);
+                        tma_load_2d(qt, &tmQKV, qf, head * D, d.rs + d.q0);
+                        tma_load_2d(qt + Cfg::kTileBytes, &tmQKV, qf, head * D, d.rs + d.q0 + 128);
                     }
                     __syncwarp();
-                    if (++st == NS) {
-                        st = 0;
-                        ph ^= 1u;
+                    for (int j = 0; j < n_max; ++j) {
+                        if (!(ok = mbar_wait_warp(&kv_empty[st], ph ^ 1u, wc, 121))) break;
+                        uint8_t* kt = smem + Cfg::kKVOff + st * 2 * Cfg::kTileBytes;
+                        if (elect_one()) {
+                            mbar_expect_tx(&kv_full[st], 2 * Cfg::kTileBytes);
+                            tma_load_2d(kt, &tmQKV, &kv_full[st], p.d_b + head * D, d.rs + d.kbase + j * 128);
+                            tma_load_2d(kt + Cfg::kTileBytes, &tmQKV, &kv_full[st], 2 * p.d_b + head * D,
+                                        d.rs + d.kbase + j * 128);
+                        }
+                        __syncwarp();
+                        if (++st == NS) {
+                            st = 0;
+                            ph ^= 1u;
+                        }
                     }
+                    if (ok && elect_one()) mbar_arrive(loads_out);
+                    __syncwarp();
                 }
-            };
-            sweep();
-            if (again(false)) {
-                sweep();
-                __syncthreads();
-                sweep();
+                ++it;   // past the end mark
+                if (!meet(pass)) break;
             }
             if (!ok) {
                 const uint64_t t0 = globaltimer();
@@ -289,136 +350,220 @@ __global__ void __launch_bounds__(kThreads, 1)
             // once P_w,j is written.  The whole warp runs the loop and computes
             // the descriptors; one elected lane issues the MMAs and commits.
             const int w = static_cast<int>(warp) - 1;
-            const int n = n_kv[w];
             // Descriptors are built once; a K=16 step adds 32 bytes (2 units of
             // 16 B) to the start address, a stage adds 2 tiles, a V step 16 rows.
             constexpr uint64_t kStageStep = (2 * Cfg::kTileBytes) >> 4;
-            const uint64_t dq = smem_desc(smem_u32(smem + Cfg::kQOff + w * Cfg::kTileBytes), 16,
-                                          Cfg::kAtomBytes, Cfg::kSwz);
+            const uint64_t dq0 = smem_desc(smem_u32(smem + Cfg::kQOff + w * Cfg::kTileBytes), 16,
+                                           Cfg::kAtomBytes, Cfg::kSwz);
             const uint64_t dk0 = smem_desc(smem_u32(smem + Cfg::kKVOff), 16, Cfg::kAtomBytes, Cfg::kSwz);
             const uint64_t dv0 = smem_desc(smem_u32(smem + Cfg::kKVOff + Cfg::kTileBytes),
                                            Cfg::kTileBytes, Cfg::kAtomBytes, Cfg::kSwz);
             const uint32_t ds = tmem_base + Cfg::kTmemS + w * 128;
             const uint32_t dout = tmem_base + Cfg::kTmemO + w * D;
             const uint32_t pa = tmem_base + Cfg::kTmemP + w * 64;
-            // ring slot and phase of tile 0 of this sweep (the producer walks n_max
-            // slots a sweep, whatever this query tile needs of them)
-            int base = 0;
-            uint32_t ns = 0, np = 0;   // S tiles read by the softmax, P tiles multiplied
-            bool ok = mbar_wait_warp(q_full, 0, wc, 221);
-            if (ok) tc_fence_after();
-            auto issue_s = [&](int j) -> bool {
-                const int g = base + j;
-                if (!mbar_wait_warp(&kv_full[g % NS], static_cast<uint32_t>(g / NS) & 1u, wc, 222)) return false;
+            // A wait that gives up leaves stale operands behind, which only this CTA's own
+            // accumulators would show; the later waits give up at once.
+            const uint32_t bar = smem_u32(&s_full[w]);
+            const bool leader = elect_one();
+            auto settle = [&](bool ready, uint32_t a, uint32_t parity, unsigned site) {
+                if (!ready) mbar_wait_slow(a, parity, wc, site);
+                __syncwarp();
                 tc_fence_after();
-                const uint64_t dk = dk0 + static_cast<uint64_t>(g % NS) * kStageStep;
-                if (elect_one()) {
+            };
+            auto wait = [&](uint64_t* b, uint32_t parity, unsigned site) {
+                const uint32_t a = smem_u32(b);
+                settle(mbar_test_wait(a, parity), a, parity, site);
+            };
+            int sl = 0;           // ring slot of the tile in hand, its phase: every role walks
+            uint32_t sp = 0;      // all n_max slots of an item
+            uint32_t ns = 0, np = 0, no = 0;   // S tiles read, P tiles multiplied, O tiles started
+            int n, n_max, sweep;
+            uint32_t it = 0, iq = 0;   // descriptors read, items (the end marks have no Q)
+            for (int pass = 0;; ++pass) {
+                for (;; ++it, ++iq) {
+                    {
+                        Item d;
+                        if (!next_item(it, &d)) break;
+                        n = w == 0 ? d.n0 : d.n1;
+                        n_max = max(d.n0, d.n1);
+                        sweep = d.sweep;
+                    }
+                    const uint64_t dq = dq0 + (iq & 1u) * ((2 * Cfg::kTileBytes) >> 4);
+                    auto issue_s = [&](int slot) {
+                        const uint64_t dk = dk0 + static_cast<uint64_t>(slot) * kStageStep;
+                        if (leader) {
 #pragma unroll
-                    for (int k = 0; k < D / 16; ++k)
-                        mma_bf16_ss(ds, dq + 2 * k, dk + 2 * k, IDESC_S, k != 0 ? 1u : 0u);
-                    mma_commit(&s_full[w]);
+                            for (int k = 0; k < D / 16; ++k)
+                                mma_bf16_ss(ds, dq + 2 * k, dk + 2 * k, IDESC_S, k != 0 ? 1u : 0u);
+                            mma_commit(&s_full[w]);
+                        }
+                        __syncwarp();
+                    };
+                    wait(&q_full[iq & 1u], (iq >> 1) & 1u, 221);
+                    if (n > 0) {
+                        wait(&kv_full[sl], sp, 222);
+                        issue_s(sl);
+                    }
+                    for (int j = 0; j < n; ++j) {
+                        const int s1 = sl + 1 == NS ? 0 : sl + 1;
+                        const uint32_t p1 = s1 == 0 ? sp ^ 1u : sp;
+                        // the next tile's operands first, so that S_w,j+1 goes out as soon as
+                        // S_w,j has been read (as it has to be before the next item's first)
+                        if (j + 1 < n) wait(&kv_full[s1], p1, 222);
+                        settle(mbar_test_wait_at<kOffFree>(bar, ns & 1u), bar + kOffFree, ns & 1u, 223);
+                        ++ns;
+                        if (j + 1 < n) {
+                            issue_s(s1);
+                        } else {
+                            if (leader) mma_commit(&q_empty[iq & 1u]);
+                            __syncwarp();
+                        }
+                        if (sweep != SWEEP_MAX) {
+                            // the item before has had its O_w read
+                            if (j == 0 && no++ > 0) wait(&o_free[w], (no - 2u) & 1u, 225);
+                            // PV in two halves of 64 keys, each issued as soon as softmax w has
+                            // written it (its V tile arrived with the K tile of S_w,j)
+                            const uint64_t dv = dv0 + static_cast<uint64_t>(sl) * kStageStep;
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const bool ready = h == 0 ? mbar_test_wait_at<kOffP0>(bar, np & 1u)
+                                                          : mbar_test_wait_at<kOffP1>(bar, np & 1u);
+                                settle(ready, bar + (h == 0 ? kOffP0 : kOffP1), np & 1u, 224);
+                                if (leader) {
+#pragma unroll
+                                    for (int q = 0; q < 4; ++q) {
+                                        // P from TMEM (16 keys = 8 columns); V: rows = keys (the K
+                                        // dimension), d contiguous (MN-major); 16 keys = two 8-row atoms.
+                                        const int kk = 4 * h + q;
+                                        mma_bf16_ts(dout, pa + kk * 8, dv + kk * ((16 * Cfg::kRowBytes) >> 4),
+                                                    IDESC_PV, (j > 0 || kk != 0) ? 1u : 0u);
+                                    }
+                                    if (h == 1) {
+                                        mma_commit(&pv_done[w]);
+                                        mma_commit(&kv_empty[sl]);
+                                    }
+                                }
+                                __syncwarp();
+                            }
+                            ++np;
+                        } else {
+                            if (leader) mma_commit(&kv_empty[sl]);
+                            __syncwarp();
+                        }
+                        sl = s1;
+                        sp = p1;
+                    }
+                    // the other query tile's key tiles past this one's: released in order,
+                    // so that no wait of this warp is ever two fills of a slot ahead
+                    if (n == 0 && leader) mbar_arrive(&q_empty[iq & 1u]);
+                    __syncwarp();
+                    for (int j = n; j < n_max; ++j) {
+                        wait(&kv_full[sl], sp, 226);
+                        if (leader) mbar_arrive(&kv_empty[sl]);
+                        __syncwarp();
+                        if (++sl == NS) {
+                            sl = 0;
+                            sp ^= 1u;
+                        }
+                    }
+                }
+                ++it;
+                if (elect_one()) mma_commit(&drain[w]);
+                __syncwarp();
+                mbar_wait_warp(&drain[w], static_cast<uint32_t>(pass), wc, 227);
+                if (!meet(pass)) break;
+            }
+        } else {
+            // ---------------------------------------------------- item scheduler
+            // The CTA's first item is its own block; once an item's loads are out, the
+            // next one is taken over from a block that has not started yet (cluster
+            // launch control), so that its first tiles load under this item's last
+            // ones.  A row sum past the limit ends the taking over; when the items in
+            // flight are done, those marked run again: row maxima, then the softmax.
+            // (one item_empty barrier per slot: a softmax group without a tile runs ahead
+            // by one item, never by two)
+            uint32_t asked = 0;   // requests made
+            auto publish = [&](uint32_t it, int bid, int sweep) -> bool {
+                const Item d = make_item(p, bid, sweep);
+                if (!mbar_wait_warp(&item_empty[it & 1u], ((it >> 1) & 1u) ^ 1u, wc, 132)) return false;
+                const int* v = reinterpret_cast<const int*>(&d);
+                if (lane == 0) {
+#pragma unroll
+                    for (int k = 0; k < kDesc; ++k) desc[(it & 1u) * kDesc + k] = v[k];
+                    mbar_arrive(&item_full[it & 1u]);
                 }
                 __syncwarp();
                 return true;
             };
-            // PV in two halves of 64 keys, each issued as soon as its softmax group
-            // has written it (its V tile arrived with the K tile of S_w,j)
-            auto issue_pv = [&](int j) -> bool {
-                const uint64_t dv = dv0 + static_cast<uint64_t>((base + j) % NS) * kStageStep;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    if (!mbar_wait_warp(&p_full[2 * w + h], np & 1u, wc, 224)) return false;
-                    tc_fence_after();
+            int bid = static_cast<int>(blockIdx.x);
+            uint32_t it = 0;
+            bool ok = true;
+            while (bid >= 0 && (ok = publish(it, bid, SWEEP_FIRST))) {
+                if (!(ok = mbar_wait_warp(loads_out, it & 1u, wc, 134))) break;
+                ++it;
+                bid = -1;
+                if (*redo_any == 0) {
                     if (elect_one()) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            // P from TMEM (16 keys = 8 columns); V: rows = keys (the K
-                            // dimension), d contiguous (MN-major); 16 keys = two 8-row atoms.
-                            const int kk = 4 * h + q;
-                            mma_bf16_ts(dout, pa + kk * 8, dv + kk * ((16 * Cfg::kRowBytes) >> 4),
-                                        IDESC_PV, (j > 0 || kk != 0) ? 1u : 0u);
-                        }
-                        if (h == 1) mma_commit(&pv_done[w]);
+                        mbar_expect_tx(clc_full, 16);
+                        clc_try_cancel(clc_answer, clc_full);
                     }
                     __syncwarp();
+                    if (!(ok = mbar_wait_warp(clc_full, asked & 1u, wc, 135))) break;
+                    ++asked;
+                    bid = clc_cancelled_block(clc_answer);
+                    fence_async_smem();   // read before the next answer overwrites it
+                    __syncwarp();
                 }
-                ++np;
-                return true;
-            };
-            // only the tiles of [0, n): the producer releases the others
-            auto sweep = [&](bool pv) {
-                if (ok && n > 0) ok = issue_s(0);
-                for (int j = 0; j < n && ok; ++j) {
-                    // S_w,j has been read before S_w,j+1 (or the next sweep's first) overwrites it
-                    ok = mbar_wait_warp(&s_free[w], ns & 1u, wc, 223);
-                    ++ns;
-                    if (!ok) break;
-                    tc_fence_after();
-                    if (j + 1 < n) ok = issue_s(j + 1);
-                    if (ok && pv) ok = issue_pv(j);
-                    if (ok) {
-                        if (elect_one()) mma_commit(&kv_empty[(base + j) % NS]);
-                        __syncwarp();
-                    }
-                }
-                base += n_max;
-            };
-            sweep(true);
-            if (again(false)) {
-                sweep(false);
-                __syncthreads();
-                sweep(true);
             }
-            if (elect_one()) mma_commit(&drain[w]);
-            __syncwarp();
-            mbar_wait_warp(&drain[w], 0, wc, 227);
-        } else if (again(false)) {
-            __syncthreads();
+            if (ok) ok = publish(it++, -1, SWEEP_FIRST);
+            if (meet(0)) {
+                for (int k = 0; k < 4 && ok; ++k) {
+                    const int again = redo[k];
+                    if (again < 0) continue;
+                    ok = publish(it, again, SWEEP_MAX) && publish(it + 1, again, SWEEP_KNOWN);
+                    it += 2;
+                }
+                if (ok) publish(it, -1, SWEEP_FIRST);
+                meet(1);
+            }
         }
     } else {
         setmaxnreg_inc<kRegsSoftmax>();
         // ---------------------------------------------------- softmax groups
         const int w = (warp >= 8) ? 1 : 0;
         const uint32_t quad = warp & 3u;
-        const int r = static_cast<int>(quad * 32 + lane);
-        const int qrow = q0 + 128 * w + r;
-        const bool valid = qrow < len;
-        // visible keys of this row, relative to the first key tile (a row past the
-        // request's end is never stored: no mask; with the running maximum it shares
-        // its warp's votes and sees one key)
-        const int cend = valid ? key_hi(p, rs, len, qrow) - kbase : (kLse ? 1 - kbase : 1 << 30);
-        const int cbeg = valid ? key_lo(p, rs, qrow) - kbase : (kLse ? -kbase : 0);
         const uint32_t lane_off = (quad * 32u) << 16;
         const uint32_t ts = tmem_base + lane_off + Cfg::kTmemS + w * 128;
         const uint32_t to = tmem_base + lane_off + Cfg::kTmemO + w * D;
         const uint32_t tp = tmem_base + lane_off + Cfg::kTmemP + w * 64;
         const float sc = p.scale_log2;
-        const int n = n_kv[w];
         float m = NEG_INF, l = 0.0f;
-        uint32_t ns = 0, np = 0;   // S tiles read, PV products waited for
-        const uint32_t a_s = smem_u32(&s_full[w]), a_free = smem_u32(&s_free[w]), a_pv = smem_u32(&pv_done[w]),
-                       a_p0 = smem_u32(&p_full[2 * w]), a_p1 = smem_u32(&p_full[2 * w + 1]);
+        uint32_t ns = 0, np = 0;         // S tiles read, P tiles written
+        int n = 0, cend = 0, cbeg = 0;   // the item's key tiles, the row's visible keys
+        const uint32_t bar = smem_u32(&s_full[w]);
         // A wait that gives up (the status word then says so) leaves stale scores
         // behind, which only this CTA's own rows would show: the loop goes on, its
         // later waits give up at once, and every role still reaches the end.
-        auto wait = [&](uint32_t a, uint32_t parity, unsigned site) {
-            if (!mbar_test_wait(a, parity)) mbar_wait_slow(a, parity, wc, site);
+        auto settle = [&](bool ready, uint32_t off, uint32_t parity, unsigned site) {
+            if (!ready) mbar_wait_slow(bar + off, parity, wc, site);
             __syncwarp();
             tc_fence_after();
         };
-        auto hand_over = [&](uint32_t a) {
+        auto hand_over = [&](auto off) {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_u32(a);
+            if (lane == 0) mbar_arrive_at<decltype(off)::value>(bar);
         };
         // the whole S row of the next tile in registers: one TMEM round trip, after
         // which the tensor core may overwrite S
-        auto take_s = [&](float (&s)[128], int j) {
-            wait(a_s, ns & 1u, 321);
+        auto take_s = [&](float (&s)[128]) {
+            settle(mbar_test_wait_at<kOffS>(bar, ns & 1u), kOffS, ns & 1u, 321);
             ++ns;
             tmem_ld64(ts, s);
             tmem_ld64(ts + 64, s + 64);
             tmem_wait_ld();
+        };
+        auto mask_s = [&](float (&s)[128], int j) {
             const int lo = cbeg - j * 128, hi = cend - j * 128;
             if (__any_sync(0xffffffffu, hi < 128 || lo > 0)) {
                 mask_chunk<0>(s, lo, hi, NEG_INF);
@@ -431,25 +576,48 @@ __global__ void __launch_bounds__(kThreads, 1)
             m = NEG_INF;
             for (int j = 0; j < n; ++j) {
                 float s[128];
-                take_s(s, j);
-                hand_over(a_free);
+                take_s(s);
+                mask_s(s, j);
+                hand_over(At<kOffFree>{});
                 m = fmaxf(m, row_max(s) * sc);
             }
+        };
+        // P of one tile (2^(s*sc - m_ref) as bf16 pairs) in two halves of 64 keys, each
+        // handed over once its store has landed.  P_w is free once PV_w of the tile
+        // before has completed: the probe's answer comes in under the second chunk's
+        // exponentials.
+        auto put_p = [&](const float (&s)[128], float m_ref, auto& rs, bool pv_waited) {
+            uint32_t pk[32];
+            exp_chunk<0>(s, sc, m_ref, pk, rs);
+            const bool pv = pv_waited || mbar_test_wait_at<kOffPV>(bar, (np & 1u) ^ 1u);
+            exp_chunk<1>(s, sc, m_ref, pk + 16, rs);
+            if (!pv_waited) settle(pv, kOffPV, (np & 1u) ^ 1u, 322);
+            ++np;
+            tmem_st32u(tp, pk);
+            tmem_wait_st();
+            hand_over(At<kOffP0>{});
+            exp_chunk<2>(s, sc, m_ref, pk, rs);
+            exp_chunk<3>(s, sc, m_ref, pk + 16, rs);
+            tmem_st32u(tp + 32, pk);
+            tmem_wait_st();
+            hand_over(At<kOffP1>{});
+        };
+        // the last PV product of an item
+        auto wait_last = [&]() {
+            settle(mbar_test_wait_at<kOffPV>(bar, (np & 1u) ^ 1u), kOffPV, (np & 1u) ^ 1u, 324);
         };
         // the training forward's form: m is the row's running maximum, moved lazily, only
         // when a tile raises it by more than 2^8 somewhere in the warp (O_w and l are
         // then rescaled)
         auto sweep_running = [&]() {
+            l = 0.0f;
             for (int j = 0; j < n; ++j) {
                 float s[128];
-                take_s(s, j);
-                hand_over(a_free);
+                take_s(s);
+                mask_s(s, j);
+                hand_over(At<kOffFree>{});
                 const float mx = row_max(s) * sc;
-                // O_w and P_w are free once PV_w,j-1 has completed
-                if (j > 0) {
-                    wait(a_pv, np & 1u, 322);
-                    ++np;
-                }
+                wait_last();   // O_w and P_w are free
                 const bool raise = (j == 0) || (mx > m + kRescaleLog2);
                 if (__any_sync(0xffffffffu, raise)) {
                     const float m_new = fmaxf(m, mx);
@@ -468,108 +636,98 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     m = m_new;
                 }
-                // (a row whose keys start in a later tile has m = -inf: its P is 0)
-                const float m_ref = (m == NEG_INF) ? 0.0f : m;
                 float rs8[8];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) rs8[q] = 0.0f;
-                uint32_t pk[32];
-                exp_chunk<0>(s, sc, m_ref, pk, rs8);
-                exp_chunk<1>(s, sc, m_ref, pk + 16, rs8);
-                tmem_st32u(tp, pk);
-                tmem_wait_st();
-                hand_over(a_p0);
-                exp_chunk<2>(s, sc, m_ref, pk, rs8);
-                exp_chunk<3>(s, sc, m_ref, pk + 16, rs8);
-                tmem_st32u(tp + 32, pk);
-                tmem_wait_st();
-                hand_over(a_p1);
+                // (a row whose keys start in a later tile has m = -inf: its P is 0)
+                put_p(s, (m == NEG_INF) ? 0.0f : m, rs8, true);
                 l += ((rs8[0] + rs8[1]) + (rs8[2] + rs8[3])) + ((rs8[4] + rs8[5]) + (rs8[6] + rs8[7]));
             }
-            if (n > 0) {
-                wait(a_pv, np & 1u, 324);
-                ++np;
-            }
+            wait_last();
         };
         // P and l of every key tile; `known`: m is the row's maximum already
         auto sweep = [&](bool known) {
-            float rs8[8];   // four pairs of running sums
-#pragma unroll
-            for (int q = 0; q < 8; ++q) rs8[q] = 0.0f;
+            float rs[2] = {0.0f, 0.0f};                // a pair of running sums
+            int fresh = known ? 0 : 1;                 // tiles before this one may find rows without reference
             for (int j = 0; j < n; ++j) {
                 float s[128];
-                take_s(s, j);
-                // rows that saw no key before take their reference here; where a row
-                // sees none yet (block-diagonal mask) m stays -inf and its P is 0
-                hand_over(a_free);
-                if (!known && __any_sync(0xffffffffu, m == NEG_INF)) {
+                take_s(s);
+                mask_s(s, j);
+                if (j < fresh) {
+                    // rows that saw no key before take their reference here; where a row
+                    // sees none yet (block-diagonal mask) m stays at kUnseen and its P is 0
                     const float mx = row_max(s) * sc;
-                    if (m == NEG_INF) m = mx;
+                    if (m == kUnseen) m = fmaxf(mx, kUnseen);
+                    if (__any_sync(0xffffffffu, m == kUnseen)) fresh = j + 2;
                 }
-                const float m_ref = (m == NEG_INF) ? 0.0f : m;
-                uint32_t pk[32];
-                exp_chunk<0>(s, sc, m_ref, pk, rs8);
-                // P_w is free once PV_w,j-1 has completed: the probe's answer comes
-                // in under the next chunk's exponentials
-                const bool pv = j > 0 && mbar_test_wait(a_pv, np & 1u);
-                exp_chunk<1>(s, sc, m_ref, pk + 16, rs8);
-                if (j > 0) {
-                    if (!pv) mbar_wait_slow(a_pv, np & 1u, wc, 322);
-                    __syncwarp();
-                    tc_fence_after();
-                    ++np;
-                }
-                tmem_st32u(tp, pk);
-                tmem_wait_st();
-                hand_over(a_p0);
-                exp_chunk<2>(s, sc, m_ref, pk, rs8);
-                exp_chunk<3>(s, sc, m_ref, pk + 16, rs8);
-                tmem_st32u(tp + 32, pk);
-                tmem_wait_st();
-                hand_over(a_p1);
+                hand_over(At<kOffFree>{});
+                put_p(s, m, rs, false);
             }
-            if (n > 0) {
-                l = ((rs8[0] + rs8[1]) + (rs8[2] + rs8[3])) + ((rs8[4] + rs8[5]) + (rs8[6] + rs8[7]));
-                wait(a_pv, np & 1u, 324);
-                ++np;
-            }
+            l = rs[0] + rs[1];
+            wait_last();
         };
-        if constexpr (kLse) {
-            sweep_running();
-            again(false);
-        } else {
-            sweep(false);
-            if (again(n > 0 && valid && !(l <= kSumLimit))) {
-                sweep_max();
-                __syncthreads();
-                sweep(true);
-            }
-        }
-        if (n > 0) {
-            const float inv = 1.0f / l;
-            // the row's log-sum-exp for a backward pass: P = 2^(s sc - (m + log2 l))
-            if (kLse && valid)
-                p.lse[static_cast<int64_t>(head) * p.req_start[p.n_req] + rs + qrow] = m + log2f(l);
-            uint16_t* dst = p.out + static_cast<int64_t>(rs + qrow) * p.d_b + head * D;
-#pragma unroll
-            for (int c = 0; c < D; c += 16) {
-                float o[16];
-                tmem_ld16(to + c, o);
-                tmem_wait_ld();
-                if (valid) {
-                    uint4* d4 = reinterpret_cast<uint4*>(dst + c);
-                    d4[0] = make_uint4(pack_bf16x2(o[0] * inv, o[1] * inv), pack_bf16x2(o[2] * inv, o[3] * inv),
-                                       pack_bf16x2(o[4] * inv, o[5] * inv), pack_bf16x2(o[6] * inv, o[7] * inv));
-                    d4[1] = make_uint4(pack_bf16x2(o[8] * inv, o[9] * inv),
-                                       pack_bf16x2(o[10] * inv, o[11] * inv),
-                                       pack_bf16x2(o[12] * inv, o[13] * inv),
-                                       pack_bf16x2(o[14] * inv, o[15] * inv));
+        // (few values live across the key tiles: the softmax threads' registers are full,
+        // and the item's descriptor stays in its slot until all of them are done with it)
+        uint32_t it = 0;
+        for (int pass = 0;; ++pass) {
+            for (bool more = true; more; ++it) {
+                const volatile Item* d = reinterpret_cast<const volatile Item*>(desc + (it & 1u) * kDesc);
+                more = mbar_wait_warp(&item_full[it & 1u], (it >> 1) & 1u, wc, 131) && d->bid >= 0;
+                n = !more ? 0 : (w == 0 ? d->n0 : d->n1);
+                if (n > 0) {
+                    // visible keys of this row, relative to the first key tile (a row past
+                    // the request's end is never stored: no mask; with the running maximum it
+                    // shares its warp's votes and sees one key)
+                    const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane), len = d->len;
+                    const int rs = d->rs, kbase = d->kbase;
+                    cend = qrow < len ? key_hi(p, rs, len, qrow) - kbase : (kLse ? 1 - kbase : 1 << 30);
+                    cbeg = qrow < len ? key_lo(p, rs, qrow) - kbase : (kLse ? -kbase : 0);
                 }
+                if (n > 0 && d->sweep == SWEEP_MAX) {
+                    sweep_max();
+                } else if (n > 0) {
+                    if (d->sweep == SWEEP_FIRST) m = kLse ? NEG_INF : kUnseen;
+                    if constexpr (kLse) sweep_running();
+                    else sweep(d->sweep == SWEEP_KNOWN);
+                    // O_w into registers, so that the next item may overwrite it
+                    float o[D];
+                    if constexpr (D == 64) {
+                        tmem_ld64(to, o);
+                    } else {
+                        tmem_ld32(to, o);
+                    }
+                    tmem_wait_ld();
+                    hand_over(At<kOffO>{});
+                    const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane);
+                    const bool valid = qrow < d->len;
+                    if (!kLse && __any_sync(0xffffffffu, valid && !(l <= kSumLimit)) && d->sweep == SWEEP_FIRST) {
+                        if (lane == 0) {
+                            redo[it & 3u] = d->bid;
+                            *redo_any = 1;
+                        }
+                    }
+                    const float inv = 1.0f / l;
+                    if (valid) {
+                        const int head = d->bid % p.n_heads;
+                        const int64_t row = d->rs + qrow;
+                        // the row's log-sum-exp for a backward pass: P = 2^(s sc - (m + log2 l))
+                        if (kLse) p.lse[static_cast<int64_t>(head) * p.req_start[p.n_req] + row] = m + log2f(l);
+                        uint4* d4 = reinterpret_cast<uint4*>(p.out + row * p.d_b + head * D);
+#pragma unroll
+                        for (int c = 0; c < D; c += 8)
+                            d4[c / 8] = make_uint4(pack_bf16x2(o[c] * inv, o[c + 1] * inv),
+                                                   pack_bf16x2(o[c + 2] * inv, o[c + 3] * inv),
+                                                   pack_bf16x2(o[c + 4] * inv, o[c + 5] * inv),
+                                                   pack_bf16x2(o[c + 6] * inv, o[c + 7] * inv));
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&item_empty[it & 1u]);
             }
+            tc_fence_before();
+            if (!meet(pass)) break;
         }
-        tc_fence_before();
     }
-    __syncthreads();
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();

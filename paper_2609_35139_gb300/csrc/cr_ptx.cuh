@@ -64,8 +64,22 @@ __device__ __forceinline__ void fence_barrier_init() {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_u32(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+// The barrier at a fixed offset from a shared-memory address.
+template <int OFF>
+__device__ __forceinline__ void mbar_arrive_at(uint32_t base) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0+%1];" ::"r"(base), "n"(OFF) : "memory");
+}
+template <int OFF>
+__device__ __forceinline__ bool mbar_test_wait_at(uint32_t base, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1+%3], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(base), "r"(parity), "n"(OFF)
+        : "memory");
+    return ok != 0;
 }
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
@@ -196,6 +210,31 @@ __device__ __forceinline__ void cluster_sync() {
 // stalled the arriving warp for about a microsecond.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+
+// Cluster launch control: ask for a block of this grid that has not started yet (its
+// launch is cancelled and its index handed over); the 16-byte answer counts on the
+// barrier.  Not to be asked again once the answer was that none is left.
+__device__ __forceinline__ void clc_try_cancel(void* answer, uint64_t* bar) {
+    asm volatile(
+        "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+            smem_u32(answer)),
+        "r"(smem_u32(bar))
+        : "memory");
+}
+// The block index (x) of an answer, or -1 if no block was left.
+__device__ __forceinline__ int clc_cancelled_block(const void* answer) {
+    int x;
+    asm volatile(
+        "{\n\t.reg .b128 h;\n\t.reg .pred q;\n\t"
+        "ld.shared.b128 h, [%1];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 q, h;\n\t"
+        "mov.b32 %0, -1;\n\t"
+        "@q clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, h;\n\t}"
+        : "=r"(x)
+        : "r"(smem_u32(answer))
+        : "memory");
+    return x;
 }
 
 // One lane of a converged warp (the lowest active one); the others get false.

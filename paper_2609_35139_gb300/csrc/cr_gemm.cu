@@ -260,7 +260,18 @@ __device__ __forceinline__ void vec16(const float* v, int col, float* out) {
 // tile, and the activations stay in L2).  n_fast: column tiles fastest, then
 // row tiles, k-parts slowest, for an A operand much larger than L2: the tiles
 // running together share their A rows and one k-range of W, so A is read once.
+// BAND (split_k = 1): the default order inside bands of band_m row tiles, one band after
+// the other (see band_rows); its own instantiations, since the extra divisions in every
+// role made the launches without bands 1 % slower.
+template <bool BAND>
 __device__ __forceinline__ int tile_lin(const GemmParams& p, int t) {
+    if constexpr (BAND) {
+        const int per = p.band_m * p.num_n;
+        const int b = t / per, r = t - b * per;
+        const int rows = min(p.band_m, p.num_m - b * p.band_m);
+        const int c = r / rows;
+        return c * p.num_m + b * p.band_m + (r - c * rows);
+    }
     if (p.n_fast) {
         const int r = t % (p.num_m * p.num_n);
         return (r % p.num_n) * p.num_m + r / p.num_n;
@@ -332,7 +343,7 @@ __device__ __forceinline__ bool named_bar_and(uint32_t id, uint32_t n, bool v) {
     return r != 0;
 }
 
-template <int BN, int EPI, int CG, int LAY>
+template <int BN, int EPI, int CG, int LAY, bool BAND>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ CUtensorMap tmC, const __grid_constant__ GemmParams p) {
@@ -430,7 +441,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         if constexpr (kPair) {
             if (reorder) return t < n_extra ? n_long + t : (t < n_extra + n_long ? t - n_extra : t);
         }
-        return tile_lin(p, t);
+        return tile_lin<BAND>(p, t);
     };
     auto k_range = [&](int t, int* kb0, int* kb1) {
         if constexpr (kPair) {
@@ -1109,11 +1120,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
 }
 
-template <int BN, int EPI, int CG, int LAY = LAY_KK>
-cr_status launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc,
-                    const GemmParams& p, cudaStream_t st) {
+template <int BN, int EPI, int CG, int LAY, bool BAND>
+cr_status launch_inst(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc,
+                      const GemmParams& p, cudaStream_t st) {
     using Cfg = GemmCfg<BN, EPI, CG>;
-    auto kern = gemm_kernel<BN, EPI, CG, LAY>;
+    auto kern = gemm_kernel<BN, EPI, CG, LAY, BAND>;
     static unsigned long long attr_done = 0;   // one per template instantiation
     const cr_status sa = ensure_smem_attr(kern, static_cast<int>(Cfg::kSmemBytes), &attr_done);
     if (sa != CR_OK) return sa;
@@ -1166,6 +1177,35 @@ cr_status launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensor
     return cuda_check(cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, p));
 }
 
+// (bands: 256-wide tiles only, the width a launch of that many rows gets)
+template <int BN, int EPI, int CG, int LAY = LAY_KK>
+cr_status launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc,
+                    const GemmParams& p, cudaStream_t st) {
+    if constexpr (BN == 256 && (LAY == LAY_KK || LAY == LAY_KK2)) {
+        if (p.band_m > 0) return launch_inst<BN, EPI, CG, LAY, true>(ta, tb, tc, p, st);
+    }
+    return launch_inst<BN, EPI, CG, LAY, false>(ta, tb, tc, p, st);
+}
+
+// Row tiles per band of the tile walk for an A operand of M x K (terms: 2 for a two-term
+// A) and a W of N x K.  W-tile-major order walks every row of A for each column tile, which
+// is free while A stays in L2 but reads a larger A from HBM once per column tile (FC2 of
+// 95617 tokens: 392 MB four times).  In bands A is read once and W once per band: one row
+// tile for a W of up to 10 MB, else about 20 MB of A.  0: A below `from` bytes, one band:
+// 64 MB, and for two products in one launch, whose tiles of unequal length are dealt out
+// in few rounds, the 128 MB of L2 (6914 tokens, 99 MB: 300 us in one band, 311 in bands).
+// Measured, us, one band / 40 MB / 20 MB / one row tile: one block of 95617 tokens at
+// d_b = 512 1458 / 1381 / 1375 / 1370; of 71889 tokens at 1024 2573 / 2237 / 2235 / 2184;
+// the 134 MB head of 48033 tokens 4187 / 4296 / 4135 / 4901; its front (W_map 16 MB)
+// 2445 / 2308 / 2226 / 2425.
+int32_t band_rows(int64_t M, int64_t N, int64_t K, int terms, int32_t num_m, int32_t num_n, double from) {
+    const double row_tile = 256.0 * static_cast<double>(K) * 2.0 * terms;
+    if (num_n < 2 || static_cast<double>(M) * static_cast<double>(K) * 2.0 * terms <= from) return 0;
+    if (static_cast<double>(N) * static_cast<double>(K) * 2.0 <= 10e6) return 1;
+    const int32_t band = static_cast<int32_t>(20e6 / row_tile);
+    return band < 1 ? 1 : (band >= num_m ? 0 : band);
+}
+
 // Every GEMM runs on CTA pairs: 256-row tiles whose MMAs span two SMs, each
 // SM loading its own 128 rows of A and half of the W tile.
 constexpr int kCG = 2;
@@ -1185,16 +1225,18 @@ cr_status launch_gemm(const uint16_t* A, int64_t lda, const uint16_t* W, int64_t
     // ceil(tiles / pairs) rounds.  Pick the instantiated width with the least
     // rounds x (256 + BN) (ties: the wider tile).  The width does not change
     // any output element's K order, so results do not depend on it.
+    // (The fp32 residual add had 160 and 128 only; with 256, O and FC2 of 95617
+    // tokens at N = 512 take 10 rounds instead of 20: the block 1590 -> 1458 us.)
     int BN;
     if (kv) {
         BN = (epi == EPI_KV_F32 || epi == EPI_KV_LOSS) ? 128 : 256;
     } else {
         const int64_t pairs = num_sms() / kCG > 0 ? num_sms() / kCG : 1;
         const int64_t mt = (M + BM * kCG - 1) / (BM * kCG);
-        static const int kF32W[] = {160, 128};
+        static const int kF32W[] = {256, 160, 128};
         static const int kBf16W[] = {256, 192, 128};
         const int* cand = f32_tile ? kF32W : kBf16W;
-        const int nc = f32_tile ? 2 : 3;
+        const int nc = 3;
         BN = cand[0];
         int64_t best = -1;
         for (int i = 0; i < nc; ++i) {
@@ -1227,6 +1269,7 @@ cr_status launch_gemm(const uint16_t* A, int64_t lda, const uint16_t* W, int64_t
     } else {
         p.col_block = 0;
     }
+    p.band_m = band_rows(M, N, K, A_lo ? 2 : 1, p.num_m, p.num_n, 64e6);
     CUtensorMap ta, tb, tc;
     if (!make_tmap_2d(&ta, A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, K, M, lda * 2, BK, BM,
                       CU_TENSOR_MAP_SWIZZLE_128B))
@@ -1262,8 +1305,9 @@ cr_status launch_gemm(const uint16_t* A, int64_t lda, const uint16_t* W, int64_t
                    : BN == 192 ? launch_bn<192, EPI_GELU_BF16, kCG>(ta, tb, tc, p, st)
                                : launch_bn<128, EPI_GELU_BF16, kCG>(ta, tb, tc, p, st);
         case EPI_ADD_F32:
-            return BN == 160 ? launch_bn<160, EPI_ADD_F32, kCG>(ta, tb, tc, p, st)
-                             : launch_bn<128, EPI_ADD_F32, kCG>(ta, tb, tc, p, st);
+            return BN == 256   ? launch_bn<256, EPI_ADD_F32, kCG>(ta, tb, tc, p, st)
+                   : BN == 160 ? launch_bn<160, EPI_ADD_F32, kCG>(ta, tb, tc, p, st)
+                               : launch_bn<128, EPI_ADD_F32, kCG>(ta, tb, tc, p, st);
         case EPI_F32:
             return BN == 256   ? launch_bn<256, EPI_F32, kCG>(ta, tb, tc, p, st)
                    : BN == 192 ? launch_bn<192, EPI_F32, kCG>(ta, tb, tc, p, st)
@@ -1357,6 +1401,7 @@ cr_status launch_gemm_pair(const GemmProduct& a, const GemmProduct& b, int64_t M
     p.n_fast = 0;
     p.col_block = 0;
     p.bgroup_rows = 0;
+    p.band_m = band_rows(M, a.N + b.N, a.K > b.K ? a.K : b.K, a.A_lo ? 2 : 1, p.num_m, p.num_n, 128e6);
     p.n_split = static_cast<int32_t>(a.N);
     p.bias = a.bias;
     p.bias2 = b.bias;
@@ -1412,6 +1457,7 @@ cr_status launch_gemm_lay(const uint16_t* A, int64_t lda, int lay, const uint16_
     p.split_kb = 0;
     p.split_k = 1;
     p.n_split = 0;
+    p.band_m = 0;
     // Split-K: when the tiles fill the CTA pairs poorly (the last round partly
     // empty), cut each tile's k-loop into s parts, each written to its own fp32
     // slice of the scratch and summed in a fixed order by a second kernel.  s

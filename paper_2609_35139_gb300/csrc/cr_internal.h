@@ -114,6 +114,9 @@ struct GemmParams {
     // tile order: 0 = W-tile-major (row tiles fastest), 1 = column tiles fastest
     // (k-parts slowest), for an A operand far larger than L2
     int32_t n_fast;
+    // > 0: the default order in bands of band_m row tiles (BAND instantiations; every
+    // launcher sets it)
+    int32_t band_m;
     // grouped rows (launch_gemm_lay): every bgroup_rows rows of A form a group whose
     // tile reads W columns [g BN, (g + 1) BN) of the W matrix, g = row / bgroup_rows,
     // and writes output columns [0, BN); 0 = off

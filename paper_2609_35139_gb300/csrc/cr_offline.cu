@@ -39,14 +39,19 @@ __device__ __forceinline__ void store8(float* p, const float* v) {
     reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
 }
 
-// One thread per (token, group of 8 rotation pairs, quarter of the layers): the
-// 8 angles q_t * f_d are computed once and applied to that group in the K
-// segments of the thread's layers (rotate-half pairs (d, d + d_h/2) inside
-// each d_h-wide segment, by -q_t f_d: (a, b) -> (a cos + b sin, b cos - a sin)),
-// one rounding to the cache dtype.  With dir = -1 the sine changes sign and the
-// rotation is by +q_t f_d, R_M itself (the stale cache's re-rotation of K to
-// request positions, Sec. 2.2).  Two segments are loaded before either is
-// rotated, for memory-level parallelism.
+// One thread per (token, layer range, KV head, group of 8 rotation pairs): the 8 angles
+// q_t * f_d are computed once and applied to that group in the head's K segment of each
+// of the thread's layers (rotate-half pairs (d, d + d_h/2) inside each d_h-wide segment,
+// by -q_t f_d: (a, b) -> (a cos + b sin, b cos - a sin)), one rounding to the cache dtype.
+// With dir = -1 the sine changes sign and the rotation is by +q_t f_d, R_M itself (the
+// stale cache's re-rotation of K to request positions, Sec. 2.2).  HBM-bound: the groups
+// and heads of one layer are neighbouring lanes, so a warp reads and writes whole runs of
+// a layer's K, and kSegs layers are loaded before any is rotated.  Measured with the
+// assembly before it (3264 tokens of the 8B shape; the rotation reads and writes 0.43
+// GB): 234 us with ranges of layers as neighbouring lanes and two segments in flight,
+// 221 with four in flight, 211 in this order with four, 206 with eight.
+constexpr int kParts = 4;   // layer ranges
+constexpr int kSegs = 8;
 template <typename T>
 __global__ void __launch_bounds__(256) canon_kernel(T* kv, int64_t n, const int32_t* __restrict__ pos,
                                                     int L, int H, int dh,
@@ -54,15 +59,17 @@ __global__ void __launch_bounds__(256) canon_kernel(T* kv, int64_t n, const int3
     pdl_launch_dependents();
     pdl_wait();
     const int groups = dh / 16;
-    constexpr int kParts = 4;   // layer ranges per (token, group)
+    const int lanes = groups * H;   // threads of one (token, layer range)
     const int64_t D = static_cast<int64_t>(2) * L * H * dh;
-    const int64_t work = n * groups * kParts;
+    const int64_t layer = static_cast<int64_t>(2) * H * dh;
+    const int64_t work = n * lanes * kParts;
     for (int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; idx < work;
          idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int part = static_cast<int>(idx % kParts);
-        const int64_t tg = idx / kParts;
-        const int64_t t = tg / groups;
-        const int g = static_cast<int>(tg - t * groups);
+        const int64_t tp = idx / lanes;
+        const int gh = static_cast<int>(idx - tp * lanes);
+        const int64_t t = tp / kParts;
+        const int part = static_cast<int>(tp - t * kParts);
+        const int h = gh / groups, g = gh - h * groups;
         const float q = static_cast<float>(__ldg(pos + t));
         float c[8], s[8];
 #pragma unroll
@@ -70,41 +77,40 @@ __global__ void __launch_bounds__(256) canon_kernel(T* kv, int64_t n, const int3
             sincos_prod(q, f.f[g * 8 + i], &s[i], &c[i]);
             s[i] *= dir;
         }
-        T* row = kv + t * D;
-        // the K segments (layer l, head h) of this part, l in [l0, l1)
-        const int l0 = part * L / kParts, l1 = (part + 1) * L / kParts;
-        const int nseg = (l1 - l0) * H;
-        for (int k = 0; k < nseg; k += 2) {
-            const int k2 = (k + 1 < nseg) ? k + 1 : k;
-            T* seg0 = row + (static_cast<int64_t>(2 * (l0 + k / H)) * H + k % H) * dh;
-            T* seg1 = row + (static_cast<int64_t>(2 * (l0 + k2 / H)) * H + k2 % H) * dh;
-            float a0[8], b0[8], a1[8], b1[8];
-            load8(seg0 + g * 8, a0);
-            load8(seg0 + dh / 2 + g * 8, b0);
-            load8(seg1 + g * 8, a1);
-            load8(seg1 + dh / 2 + g * 8, b1);
+        const int l1 = (part + 1) * L / kParts;
+        T* const first = kv + t * D + h * dh + g * 8;
+        for (int l = part * L / kParts; l < l1; l += kSegs) {
+            float a[kSegs][8], b[kSegs][8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float x0 = a0[i], y0 = b0[i], x1 = a1[i], y1 = b1[i];
-                a0[i] = x0 * c[i] + y0 * s[i];
-                b0[i] = y0 * c[i] - x0 * s[i];
-                a1[i] = x1 * c[i] + y1 * s[i];
-                b1[i] = y1 * c[i] - x1 * s[i];
+            for (int u = 0; u < kSegs; ++u) {
+                const T* p = first + (l + u < l1 ? l + u : l) * layer;
+                load8(p, a[u]);
+                load8(p + dh / 2, b[u]);
             }
-            store8(seg0 + g * 8, a0);
-            store8(seg0 + dh / 2 + g * 8, b0);
-            if (k2 != k) {
-                store8(seg1 + g * 8, a1);
-                store8(seg1 + dh / 2 + g * 8, b1);
+#pragma unroll
+            for (int u = 0; u < kSegs; ++u) {
+                if (l + u >= l1) break;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float x = a[u][i], y = b[u][i];
+                    a[u][i] = x * c[i] + y * s[i];
+                    b[u][i] = y * c[i] - x * s[i];
+                }
+                T* p = first + (l + u) * layer;
+                store8(p, a[u]);
+                store8(p + dh / 2, b[u]);
             }
         }
     }
 }
 
-// Partial sums of squares: block (x, y) covers 2048 coordinates (8 per thread)
-// over the 64-token slice y; part[y][j].  With b, the squares of a - b.
+// Partial sums of squares: block (x, y) covers 1024 coordinates (8 per thread)
+// over the 64-token slice y; part[y][j].  With b, the squares of a - b.  HBM-bound:
+// blocks of 128 threads leave less of the chip idle in the last round than 256 (4096
+// tokens of the 7B shape against another cache, 0.47 GB: the statistic 107 -> 92 us).
+constexpr int kSigmaThreads = 128;
 template <typename T>
-__global__ void __launch_bounds__(256) sigma_partial_kernel(const T* __restrict__ a, const T* __restrict__ b,
+__global__ void __launch_bounds__(kSigmaThreads) sigma_partial_kernel(const T* __restrict__ a, const T* __restrict__ b,
                                                             int64_t n, int64_t D, float* __restrict__ part) {
     pdl_launch_dependents();
     pdl_wait();
@@ -148,15 +154,27 @@ __global__ void __launch_bounds__(256) sigma_partial_kernel(const T* __restrict_
     store8(part + static_cast<int64_t>(blockIdx.y) * D + col, acc);
 }
 
-// sumsq[j] += sum over slices, in slice order (deterministic), in fp64.
+// sumsq[j] += sum over slices, in slice order (deterministic), in fp64.  A chain of loads:
+// sixteen slices in flight and blocks of 64 threads, so that every SM has some (111 ->
+// 107 us of the statistic above).
 __global__ void __launch_bounds__(256) sigma_reduce_kernel(const float* __restrict__ part, int slices,
                                                            int64_t D, double* sumsq) {
     pdl_launch_dependents();
     pdl_wait();
     for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j < D;
          j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        // sixteen slices in flight, added in slice order
         double s = 0.0;
-        for (int k = 0; k < slices; ++k) s += static_cast<double>(part[static_cast<int64_t>(k) * D + j]);
+        const float* p = part + j;
+        int k = 0;
+        for (; k + 16 <= slices; k += 16) {
+            float v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = p[(k + u) * D];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) s += static_cast<double>(v[u]);
+        }
+        for (; k < slices; ++k) s += static_cast<double>(p[k * D]);
         sumsq[j] += s;
     }
 }
@@ -178,7 +196,7 @@ cr_status launch_canonicalize(void* kv, bool f32, int64_t n, const int32_t* pos,
     if (dh != 64 && dh != 128) return CR_ERR_UNSUPPORTED;
     Freq f{};
     for (int i = 0; i < dh / 2; ++i) f.f[i] = inv_freq_host[i];
-    const int64_t work = n * (dh / 16) * 4;
+    const int64_t work = n * (dh / 16) * H * kParts;
     int64_t blocks = (work + 255) / 256;
     if (blocks > static_cast<int64_t>(num_sms()) * 16) blocks = static_cast<int64_t>(num_sms()) * 16;
     const dim3 grid(static_cast<unsigned>(blocks)), block(256);
@@ -193,18 +211,17 @@ cr_status launch_sigma_accumulate(const void* a, const void* b, bool f32, int64_
                                   float* part, double* sumsq, cudaStream_t st) {
     if (n <= 0) return CR_OK;
     const int64_t slices = (n + kSigmaSlice - 1) / kSigmaSlice;
-    const dim3 grid(static_cast<unsigned>((D / 8 + 255) / 256), static_cast<unsigned>(slices));
+    const dim3 grid(static_cast<unsigned>((D / 8 + kSigmaThreads - 1) / kSigmaThreads), static_cast<unsigned>(slices));
     cr_status s;
     if (f32)
-        s = launch_pdl(sigma_partial_kernel<float>, grid, dim3(256), 0, st, static_cast<const float*>(a),
+        s = launch_pdl(sigma_partial_kernel<float>, grid, dim3(kSigmaThreads), 0, st, static_cast<const float*>(a),
                        static_cast<const float*>(b), n, D, part);
     else
-        s = launch_pdl(sigma_partial_kernel<uint16_t>, grid, dim3(256), 0, st,
+        s = launch_pdl(sigma_partial_kernel<uint16_t>, grid, dim3(kSigmaThreads), 0, st,
                        static_cast<const uint16_t*>(a), static_cast<const uint16_t*>(b), n, D, part);
     if (s != CR_OK) return s;
-    int64_t blocks = (D + 255) / 256;
-    if (blocks > static_cast<int64_t>(num_sms()) * 8) blocks = static_cast<int64_t>(num_sms()) * 8;
-    return launch_pdl(sigma_reduce_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, st,
+    const int64_t blocks = (D + 63) / 64;
+    return launch_pdl(sigma_reduce_kernel, dim3(static_cast<unsigned>(blocks)), dim3(64), 0, st,
                       static_cast<const float*>(part), static_cast<int>(slices), D, sumsq);
 }
 

@@ -199,11 +199,12 @@ __device__ __forceinline__ Item make_item(const AttnParams& p, int bid, int swee
     return d;
 }
 
-// kLse: the training forward.  It also writes each row's log-sum-exp (for the
-// backward), and it keeps the running maximum as reference: P's bf16 rounding depends
-// on the reference, and a training step amplifies such a change into 2e-3 of its fp32
-// gradients' norm after six blocks, so its results stay bit for bit what they were.
-template <int D, bool kLse>
+// kRunning: the reference is the running maximum.  P's bf16 rounding depends on the
+// reference, and fp32 results show it: a training step amplifies the change into 2e-3 of
+// its fp32 gradients' norm after six blocks, an fp32 cache moves by 1e-4.  So the training
+// forward, which also writes each row's log-sum-exp for the backward, and the forward of
+// fp32 caches keep the running maximum, and their results stay bit for bit what they were.
+template <int D, bool kRunning>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_constant__ AttnParams p) {
     using Cfg = AttnCfg<D>;
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // they walk the items to run again.
     auto meet = [&](int pass) -> bool {
         __syncthreads();
-        return !kLse && pass == 0 && *redo_any != 0;
+        return !kRunning && pass == 0 && *redo_any != 0;
     };
     // The descriptor of the CTA's it-th item, for the producer and issuer warps; false at
     // the end (or when a role has given up).
@@ -606,7 +607,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         auto wait_last = [&]() {
             settle(mbar_test_wait_at<kOffPV>(bar, (np & 1u) ^ 1u), kOffPV, (np & 1u) ^ 1u, 324);
         };
-        // the training forward's form: m is the row's running maximum, moved lazily, only
+        // the kRunning form: m is the row's running maximum, moved lazily, only
         // when a tile raises it by more than 2^8 somewhere in the warp (O_w and l are
         // then rescaled)
         auto sweep_running = [&]() {
@@ -680,14 +681,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // shares its warp's votes and sees one key)
                     const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane), len = d->len;
                     const int rs = d->rs, kbase = d->kbase;
-                    cend = qrow < len ? key_hi(p, rs, len, qrow) - kbase : (kLse ? 1 - kbase : 1 << 30);
-                    cbeg = qrow < len ? key_lo(p, rs, qrow) - kbase : (kLse ? -kbase : 0);
+                    cend = qrow < len ? key_hi(p, rs, len, qrow) - kbase : (kRunning ? 1 - kbase : 1 << 30);
+                    cbeg = qrow < len ? key_lo(p, rs, qrow) - kbase : (kRunning ? -kbase : 0);
                 }
                 if (n > 0 && d->sweep == SWEEP_MAX) {
                     sweep_max();
                 } else if (n > 0) {
-                    if (d->sweep == SWEEP_FIRST) m = kLse ? NEG_INF : kUnseen;
-                    if constexpr (kLse) sweep_running();
+                    if (d->sweep == SWEEP_FIRST) m = kRunning ? NEG_INF : kUnseen;
+                    if constexpr (kRunning) sweep_running();
                     else sweep(d->sweep == SWEEP_KNOWN);
                     // O_w into registers, so that the next item may overwrite it
                     float o[D];
@@ -700,7 +701,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     hand_over(At<kOffO>{});
                     const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane);
                     const bool valid = qrow < d->len;
-                    if (!kLse && __any_sync(0xffffffffu, valid && !(l <= kSumLimit)) && d->sweep == SWEEP_FIRST) {
+                    if (!kRunning && __any_sync(0xffffffffu, valid && !(l <= kSumLimit)) && d->sweep == SWEEP_FIRST) {
                         if (lane == 0) {
                             redo[it & 3u] = d->bid;
                             *redo_any = 1;
@@ -711,7 +712,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const int head = d->bid % p.n_heads;
                         const int64_t row = d->rs + qrow;
                         // the row's log-sum-exp for a backward pass: P = 2^(s sc - (m + log2 l))
-                        if (kLse) p.lse[static_cast<int64_t>(head) * p.req_start[p.n_req] + row] = m + log2f(l);
+                        if (kRunning && p.lse)
+                            p.lse[static_cast<int64_t>(head) * p.req_start[p.n_req] + row] = m + log2f(l);
                         uint4* d4 = reinterpret_cast<uint4*>(p.out + row * p.d_b + head * D);
 #pragma unroll
                         for (int c = 0; c < D; c += 8)
@@ -735,10 +737,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-template <int D, bool kLse>
+template <int D, bool kRunning>
 cr_status launch_d(const CUtensorMap& tm, const AttnParams& p, cudaStream_t st) {
     using Cfg = AttnCfg<D>;
-    auto kern = attn_kernel<D, kLse>;
+    auto kern = attn_kernel<D, kRunning>;
     static unsigned long long attr_done = 0;   // one per template instantiation
     const cr_status sa = ensure_smem_attr(kern, static_cast<int>(Cfg::kSmemBytes), &attr_done);
     if (sa != CR_OK) return sa;
@@ -808,7 +810,7 @@ cr_status launch_attention(const uint16_t* qkv, int64_t n_tokens, int head_dim,
                       3ull * p.d_b * 2, head_dim, 128,
                       head_dim == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
         return CR_ERR_INVALID_ARG;
-    if (p.lse) return head_dim == 64 ? launch_d<64, true>(tm, p, st) : launch_d<32, true>(tm, p, st);
+    if (p.lse || p.running) return head_dim == 64 ? launch_d<64, true>(tm, p, st) : launch_d<32, true>(tm, p, st);
     return head_dim == 64 ? launch_d<64, false>(tm, p, st) : launch_d<32, false>(tm, p, st);
 }
 

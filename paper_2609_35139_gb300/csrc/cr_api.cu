@@ -1155,7 +1155,7 @@ cr_status cr_param_layout(const cr_target_dims* target, const cr_repairer_dims* 
 namespace {
 struct TrainLayout {
     size_t inf, h0, rein, blk, blk_stride, hbuf, yf, rope, dz, rowsq, rowscale, losspart, perreq,
-        stats_pad, dh, dxm, du, dtmp, pre, gprod, sig16, dqkv, da, lse, dvec, cstart, dse, dy, colsum, colcnt,
+        stats_pad, dh, dxm, du, dtmp, pre, sig16, dqkv, da, lse, dvec, cstart, dse, dy, colsum, colcnt,
         norm, segw, splitk, total;
     size_t x_in, x_mid, u1, u2, qkv, o, g;   // offsets inside one block's region
 };
@@ -1202,7 +1202,6 @@ TrainLayout train_layout(const Dims& d, int64_t n) {
     const int64_t wide = std::max(std::max(d.hid, 3 * d.db), std::max(2 * d.dc, d.S * d.dseg));
     L.dtmp = take(N * d.hid * 4);
     L.pre = take(N * d.hid * 4);
-    L.gprod = take(N * d.db * 4);
     L.sig16 = take(N * wide * 2);
     L.dqkv = take(N * 3 * d.db * 4);
     L.da = take(N * d.db * 4);
@@ -1215,7 +1214,9 @@ TrainLayout train_layout(const Dims& d, int64_t n) {
     L.colcnt = take(colsum_counters(std::max(d.D, wide)) * 4);
     L.norm = take(sqnorm_scratch_doubles() * 8);
     L.segw = take(static_cast<size_t>(d.D) * 128 * 4);   // grouped W_seg gradient blocks
-    L.splitk = take(8 * N * d.db * 4);                     // split-K parts of the backward's products
+    // split-K parts of the backward's products; between them the LayerNorm backward's partial sums
+    L.splitk = take(std::max(8 * N * static_cast<size_t>(d.db),
+                             ln_backward_scratch_floats(n, static_cast<int>(d.db))) * 4);
     L.total = off;
     return L;
 }
@@ -1268,6 +1269,8 @@ cr_status cr_train_step(const cr_target_dims* target, const cr_repairer_dims* re
     int64_t off[14 + 12 * 64 + 1];
     const int nt = train_offsets(d, off, 14 + 12 * 64 + 1);
     if (nt < 0) return CR_ERR_INVALID_ARG;
+    int64_t sizes[14 + 12 * 64];
+    train_tensor_sizes(d, sizes, 14 + 12 * 64);
     const int64_t P = off[nt];
     unsigned* status = device_status_ptr();
     if (!status) return CR_ERR_CUDA;
@@ -1342,7 +1345,6 @@ cr_status cr_train_step(const cr_target_dims* target, const cr_repairer_dims* re
     float* DU = at<float>(base, L.du);
     float* DTMP = at<float>(base, L.dtmp);
     float* PRE = at<float>(base, L.pre);
-    float* GPROD = at<float>(base, L.gprod);
     uint16_t* SIG = at<uint16_t>(base, L.sig16);
     float* DQKV = at<float>(base, L.dqkv);
     float* DA = at<float>(base, L.da);
@@ -1402,8 +1404,10 @@ cr_status cr_train_step(const cr_target_dims* target, const cr_repairer_dims* re
         uint16_t* qkv = reinterpret_cast<uint16_t*>(blk(b, L.qkv));
         uint16_t* o = reinterpret_cast<uint16_t*>(blk(b, L.o));
         uint16_t* g = reinterpret_cast<uint16_t*>(blk(b, L.g));
+        // (x_mid and H start as copies of what their LayerNorm read: the residual adds below
+        // are in place)
         if ((s = launch_layernorm(b == 0 ? h0 : H, rein + b * db, B * db, x_in, k.ln1_g, k.ln1_b, eps, N, db,
-                                  u1, st)) != CR_OK)
+                                  u1, st, x_mid)) != CR_OK)
             break;
         gq.bias = k.b_qkv;
         gq.out = qkv;
@@ -1412,22 +1416,16 @@ cr_status cr_train_step(const cr_target_dims* target, const cr_repairer_dims* re
         ap->out = o;
         ap->lse = LSE + b * d.nh * N;
         if ((s = launch_attention(qkv, N, static_cast<int>(hd), *ap, st)) != CR_OK) break;
-        if ((s = cuda_check(cudaMemcpyAsync(x_mid, x_in, static_cast<size_t>(N * db) * 4,
-                                            cudaMemcpyDeviceToDevice, st))) != CR_OK)
-            break;
         gr.bias = k.b_o;
         gr.out = x_mid;
         gr.ldo = db;
         if ((s = launch_gemm(o, db, k.w_o, N, db, db, EPI_ADD_F32, gr, nullptr, 0, st)) != CR_OK) break;
-        if ((s = launch_layernorm(x_mid, nullptr, 0, nullptr, k.ln2_g, k.ln2_b, eps, N, db, u2, st)) != CR_OK)
+        if ((s = launch_layernorm(x_mid, nullptr, 0, nullptr, k.ln2_g, k.ln2_b, eps, N, db, u2, st, H)) != CR_OK)
             break;
         gr.bias = k.b_fc1;
         gr.out = g;
         gr.ldo = hid;
         if ((s = launch_gemm(u2, db, k.w_fc1, N, hid, db, EPI_GELU_BF16, gr, nullptr, 0, st)) != CR_OK) break;
-        if ((s = cuda_check(cudaMemcpyAsync(H, x_mid, static_cast<size_t>(N * db) * 4,
-                                            cudaMemcpyDeviceToDevice, st))) != CR_OK)
-            break;
         gr.bias = k.b_fc2;
         gr.out = H;
         gr.ldo = db;
@@ -1457,7 +1455,13 @@ cr_status cr_train_step(const cr_target_dims* target, const cr_repairer_dims* re
     if (s != CR_OK) return s;
 
     // ---- backward: the chain rule in reverse, gradients straight into `grads`
-    if ((s = cuda_check(cudaMemsetAsync(grads, 0, static_cast<size_t>(P) * 4, st))) != CR_OK) return s;
+    // (every tensor's gradient is written whole; only the gaps between tensors are cleared:
+    // clearing all 600 MB of the 8B shape's took 90 us)
+    for (int k = 0; k < nt; ++k)
+        if (off[k] + sizes[k] < off[k + 1] &&
+            (s = cuda_check(cudaMemsetAsync(grads + off[k] + sizes[k], 0,
+                                            static_cast<size_t>(off[k + 1] - off[k] - sizes[k]) * 4, st))) != CR_OK)
+            return s;
     // column-sum election counters start at zero (each use leaves them at zero)
     if ((s = cuda_check(cudaMemsetAsync(CCNT, 0, colsum_counters(std::max(d.D, std::max(std::max(d.hid, 3 * d.db),
                                                                            std::max(2 * d.dc, d.S * d.dseg)))) *
@@ -1491,9 +1495,11 @@ cr_status cr_train_step(const cr_target_dims* target, const cr_repairer_dims* re
     CR_TRY(mm(DZ, D, true, yf, db, D, db, N, gk(W_OUT), db, false));
     CR_TRY(colsum(DZ, true, D, D, gk(B_OUT)));
     CR_TRY(mm(DZ, D, false, pb(W_OUT), db, N, db, D, DU, db, false));
-    CR_TRY(launch_ln_backward(H, w.lnf_g, DU, nullptr, eps, N, static_cast<int>(db), DH, GPROD, st));
-    CR_TRY(colsum(GPROD, false, db, db, gk(LNFG)));
-    CR_TRY(colsum(DU, false, db, db, gk(LNFB)));
+    // A LayerNorm's backward leaves dx in fp32 (DH, DXM) and, for the products that follow,
+    // in bf16 (SIG), with dx's column sums: the bias gradient of the linear whose output
+    // the LayerNorm read, and (DH) of the reinjection or the fusion that was added to it.
+    CR_TRY(launch_ln_backward(H, w.lnf_g, DU, nullptr, eps, N, static_cast<int>(db), DH, SIG, gk(LNFG), gk(LNFB),
+                              B > 0 ? gk(bk(B - 1, BFC2)) : gk(B_FUSE), nullptr, SPLITK, st));
     CR_TRY(cuda_check(cudaMemsetAsync(DSE, 0, static_cast<size_t>(N * 2 * dc) * 4, st)));
     for (int64_t b = B - 1; b >= 0; --b) {
         const float* x_in = reinterpret_cast<const float*>(blk(b, L.x_in));
@@ -1504,7 +1510,6 @@ cr_status cr_train_step(const cr_target_dims* target, const cr_repairer_dims* re
         const uint16_t* o = reinterpret_cast<const uint16_t*>(blk(b, L.o));
         const uint16_t* g = reinterpret_cast<const uint16_t*>(blk(b, L.g));
         // h = x_mid + W_fc2 g + b_fc2
-        CR_TRY(colsum16(DH, db, SIG, gk(bk(b, BFC2))));
         CR_TRY(mm(SIG, db, true, g, hid, db, hid, N, gk(bk(b, WFC2)), hid, false));
         CR_TRY(mm(SIG, db, false, pb(bk(b, WFC2)), hid, N, hid, db, DTMP, hid, false));
         // g = GELU(pre), pre = W_fc1 u2 + b_fc1 (recomputed in fp32)
@@ -1514,39 +1519,33 @@ cr_status cr_train_step(const cr_target_dims* target, const cr_repairer_dims* re
         gp.out = PRE;
         gp.ldo = hid;
         CR_TRY(launch_gemm(u2, db, pb(bk(b, WFC1)), N, hid, db, EPI_F32, gp, nullptr, 0, st));
-        CR_TRY(launch_gelu_backward(DTMP, PRE, N * hid, st));
-        CR_TRY(colsum16(DTMP, hid, SIG, gk(bk(b, BFC1))));
+        CR_TRY(launch_gelu_backward(DTMP, PRE, N, hid, SIG, gk(bk(b, BFC1)), CS, CCNT, st));
         CR_TRY(mm(SIG, hid, true, u2, db, hid, db, N, gk(bk(b, WFC1)), db, false));
         CR_TRY(mm(SIG, hid, false, pb(bk(b, WFC1)), db, N, db, hid, DU, db, false));
         // u2 = LN2(x_mid): dx_mid = dh + LN2 backward
-        CR_TRY(launch_ln_backward(x_mid, pf(bk(b, LN2G)), DU, DH, eps, N, static_cast<int>(db), DXM, GPROD, st));
-        CR_TRY(colsum(GPROD, false, db, db, gk(bk(b, LN2G))));
-        CR_TRY(colsum(DU, false, db, db, gk(bk(b, LN2B))));
+        CR_TRY(launch_ln_backward(x_mid, pf(bk(b, LN2G)), DU, DH, eps, N, static_cast<int>(db), DXM, SIG,
+                                  gk(bk(b, LN2G)), gk(bk(b, LN2B)), gk(bk(b, BO)), nullptr, SPLITK, st));
         // x_mid = x_in + W_o a + b_o
-        CR_TRY(colsum16(DXM, db, SIG, gk(bk(b, BO))));
         CR_TRY(mm(SIG, db, true, o, db, db, db, N, gk(bk(b, WO)), db, false));
         CR_TRY(mm(SIG, db, false, pb(bk(b, WO)), db, N, db, db, DA, db, false));
         // attention: the fused backward (P recomputed from the forward's log-sum-exp,
         // dQ, dK, dV into dqkv), dO in bf16 for its MMAs
-        CR_TRY(to16(DA, N * db, SIG));
         bp->lse = LSE + b * d.nh * N;
         bp->dqkv = DQKV;
         CR_TRY(launch_attention_backward(qkv, SIG, DA, o, N, static_cast<int>(hd), *bp, DVEC, st));
-        CR_TRY(launch_rope_backward(DQKV, rope, N, static_cast<int>(db), static_cast<int>(hd), st));
         // qkv = W_qkv u1 + b_qkv;  u1 = LN1(x_in): dx_in = dx_mid + LN1 backward
-        CR_TRY(colsum16(DQKV, 3 * db, SIG, gk(bk(b, BQKV))));
+        CR_TRY(launch_rope_backward(DQKV, rope, N, static_cast<int>(db), static_cast<int>(hd), SIG,
+                                    gk(bk(b, BQKV)), CS, CCNT, st));
         CR_TRY(mm(SIG, 3 * db, true, u1, db, 3 * db, db, N, gk(bk(b, WQKV)), db, false));
         CR_TRY(mm(SIG, 3 * db, false, pb(bk(b, WQKV)), db, N, db, 3 * db, DU, db, false));
-        CR_TRY(launch_ln_backward(x_in, pf(bk(b, LN1G)), DU, DXM, eps, N, static_cast<int>(db), DH, GPROD, st));
-        CR_TRY(colsum(GPROD, false, db, db, gk(bk(b, LN1G))));
-        CR_TRY(colsum(DU, false, db, db, gk(bk(b, LN1B))));
+        CR_TRY(launch_ln_backward(x_in, pf(bk(b, LN1G)), DU, DXM, eps, N, static_cast<int>(db), DH, SIG,
+                                  gk(bk(b, LN1G)), gk(bk(b, LN1B)), gk(B_REIN) + b * db,
+                                  b > 0 ? gk(bk(b - 1, BFC2)) : gk(B_FUSE), SPLITK, st));
         // x_in = h^{b-1} + W_rein,b s + b_rein,b: ds += dx_in W_rein,b
-        CR_TRY(colsum16(DH, db, SIG, gk(B_REIN) + b * db));
         CR_TRY(mm(SIG, db, true, se, 4 * dc, db, dc, N, gk(W_REIN) + b * db * dc, dc, false));
         CR_TRY(mm(SIG, db, false, pb(W_REIN) + b * db * dc, dc, N, dc, db, DSE, 2 * dc, true));
     }
     // h0 = W_fuse [s; e] + b_fuse
-    CR_TRY(colsum16(DH, db, SIG, gk(B_FUSE)));
     CR_TRY(mm(SIG, db, true, se, 4 * dc, db, 2 * dc, N, gk(W_FUSE), 2 * dc, false));
     CR_TRY(mm(SIG, db, false, pb(W_FUSE), 2 * dc, N, 2 * dc, db, DSE, 2 * dc, true));
     // e = W_tok emb + b_tok;  s = W_map y + b_map

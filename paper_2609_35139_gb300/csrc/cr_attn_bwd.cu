@@ -442,10 +442,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
     }
 }
 
-// D[h][t] = sum_d dO[t, h d + d] O[t, h d + d]: one thread per (token, head)
+// D[h][t] = sum_d dO[t, h d + d] O[t, h d + d]: one thread per (token, head); dO's bf16
+// copy is written from the same read
 __global__ void __launch_bounds__(256)
     attn_bwd_dvec_kernel(const float* __restrict__ dO, const uint16_t* __restrict__ O, int64_t N, int db, int hd,
-                         float* __restrict__ dvec) {
+                         float* __restrict__ dvec, uint16_t* __restrict__ dO16) {
     pdl_launch_dependents();
     pdl_wait();
     const int heads = db / hd;
@@ -460,6 +461,9 @@ __global__ void __launch_bounds__(256)
         const uint4 w = *reinterpret_cast<const uint4*>(o + k);
         const float4 x0 = *reinterpret_cast<const float4*>(a + k);
         const float4 x1 = *reinterpret_cast<const float4*>(a + k + 4);
+        *reinterpret_cast<uint4*>(dO16 + t * db + h * hd + k) =
+            make_uint4(pack_bf16x2(x0.x, x0.y), pack_bf16x2(x0.z, x0.w), pack_bf16x2(x1.x, x1.y),
+                       pack_bf16x2(x1.z, x1.w));
         s = fmaf(x0.x, __uint_as_float(w.x << 16), s);
         s = fmaf(x0.y, __uint_as_float(w.x & 0xFFFF0000u), s);
         s = fmaf(x0.z, __uint_as_float(w.y << 16), s);
@@ -487,13 +491,13 @@ cr_status launch_bwd_d(const CUtensorMap& tq, const CUtensorMap& td, const AttnB
 
 }  // namespace
 
-cr_status launch_attention_backward(const uint16_t* qkv, const uint16_t* dO16, const float* dO, const uint16_t* O,
+cr_status launch_attention_backward(const uint16_t* qkv, uint16_t* dO16, const float* dO, const uint16_t* O,
                                     int64_t n_tokens, int head_dim, AttnBwdParams& p, float* dvec, cudaStream_t st) {
     if (head_dim != 32 && head_dim != 64) return CR_ERR_UNSUPPORTED;
     if (p.n_items <= 0) return CR_OK;
     const int64_t pairs = n_tokens * (p.d_b / head_dim);
     cr_status s = launch_pdl(attn_bwd_dvec_kernel, dim3(static_cast<unsigned>((pairs + 255) / 256)), dim3(256), 0,
-                             st, dO, O, n_tokens, p.d_b, head_dim, dvec);
+                             st, dO, O, n_tokens, p.d_b, head_dim, dvec, dO16);
     if (s != CR_OK) return s;
     p.dvec = dvec;
     CUtensorMap tq, td;

@@ -329,16 +329,18 @@ cr_status launch_split_bf16(const float* x, int64_t rows, int64_t cols, uint16_t
                             cudaStream_t st);
 cr_status launch_rope_table(const int32_t* pos, int64_t n, int half_dim, const float* inv_freq_host,
                             float2* table, cudaStream_t st);
+// x_copy (optional): the normalised row x (+ add) once more, for a residual add in place.
 cr_status launch_layernorm(const float* x, const float* add, int64_t ld_add, float* x_out,
                            const float* g, const float* b, float eps, int64_t M, int64_t D,
-                           uint16_t* u, cudaStream_t st);
+                           uint16_t* u, cudaStream_t st, float* x_copy = nullptr);
 cr_status launch_wait_selftest(unsigned* status, cudaStream_t st);
 cr_status launch_chunk_starts(const int32_t* chunk_end, const AttnParams& p, int64_t n_tokens,
                               int32_t* chunk_start, cudaStream_t st);
 cr_status launch_attention(const uint16_t* qkv, int64_t n_tokens, int head_dim,
                            const AttnParams& p, cudaStream_t st);
 
-cr_status launch_attention_backward(const uint16_t* qkv, const uint16_t* dO16, const float* dO, const uint16_t* O,
+// dO16 [N, d_b] receives dO rounded to bf16 (the MMAs' operand).
+cr_status launch_attention_backward(const uint16_t* qkv, uint16_t* dO16, const float* dO, const uint16_t* O,
                                     int64_t n_tokens, int head_dim, AttnBwdParams& p, float* dvec, cudaStream_t st);
 
 // training step (cr_train.cu)
@@ -359,10 +361,18 @@ cr_status launch_colsum_bf16(const float* a, int64_t rows, int64_t cols, uint16_
                              float* scratch, unsigned* counters, cudaStream_t st);
 cr_status launch_colsum(const void* a, bool bf16, int64_t rows, int64_t cols, int64_t lda, float* out,
                         bool accumulate, float* scratch, unsigned* counters, cudaStream_t st);
+// LayerNorm backward: dx (fp32 and bf16), the parameter gradients, and dx's column sums
+// (a bias gradient) into dbias and, if given, dbias2; scratch: ln_backward_scratch_floats.
+size_t ln_backward_scratch_floats(int64_t N, int D);
 cr_status launch_ln_backward(const float* x, const float* gamma, const float* dy, const float* add, float eps,
-                             int64_t N, int D, float* dx, float* gprod, cudaStream_t st);
-cr_status launch_gelu_backward(float* dg, const float* pre, int64_t n, cudaStream_t st);
-cr_status launch_rope_backward(float* dqkv, const float2* table, int64_t N, int db, int hd, cudaStream_t st);
+                             int64_t N, int D, float* dx, uint16_t* dx16, float* dgamma, float* dbeta, float* dbias,
+                             float* dbias2, float* scratch, cudaStream_t st);
+// dg * GELU'(pre) and the RoPE transpose of dqkv [N, 3 d_b], each rounded to bf16 into a16
+// with its column sums into out (as launch_colsum_bf16).
+cr_status launch_gelu_backward(const float* dg, const float* pre, int64_t rows, int64_t cols, uint16_t* a16,
+                               float* out, float* scratch, unsigned* counters, cudaStream_t st);
+cr_status launch_rope_backward(const float* dqkv, const float2* table, int64_t N, int db, int hd, uint16_t* a16,
+                               float* out, float* scratch, unsigned* counters, cudaStream_t st);
 // The W_seg gradient from the grouped dW GEMM's blocks ([S d_h, 128] fp32, the
 // rows of segment s carrying its d_seg columns at (s mod (128 / d_seg)) d_seg):
 // g [S][d_seg][d_h] = block / sigma_stale (the fold of 1/sigma into W_seg).

@@ -133,7 +133,8 @@ __global__ void __launch_bounds__(256) layernorm_kernel(const float* x,
                                                         int64_t ld_add, float* x_out,
                                                         const float* __restrict__ g,
                                                         const float* __restrict__ b, float eps,
-                                                        int64_t M, uint16_t* __restrict__ u) {
+                                                        int64_t M, uint16_t* __restrict__ u,
+                                                        float* x_copy) {
     constexpr int D = VPL * 128;
     constexpr int HV = VPL / WPR;            // float4 per lane
     constexpr int RPB = 8 / WPR;             // rows per CTA
@@ -166,6 +167,11 @@ __global__ void __launch_bounds__(256) layernorm_kernel(const float* x,
             v[k].w += av[k].w;
             if (live) xo[lane + 32 * k] = v[k];
         }
+    }
+    if (x_copy && live) {
+        float4* xc = reinterpret_cast<float4*>(x_copy + rr * D) + c0;
+#pragma unroll
+        for (int k = 0; k < HV; ++k) xc[lane + 32 * k] = v[k];
     }
     // the row's sum over its WPR warps (the same order in every warp of the row)
     auto row_sum = [&](float s, int slot) {
@@ -352,7 +358,7 @@ cr_status launch_gather(const GatherParams& p, cudaStream_t st) {
 
 cr_status launch_layernorm(const float* x, const float* add, int64_t ld_add, float* x_out,
                            const float* g, const float* b, float eps, int64_t M, int64_t D,
-                           uint16_t* u, cudaStream_t st) {
+                           uint16_t* u, cudaStream_t st, float* x_copy) {
     if (M <= 0) return CR_OK;
     switch (D) {
 #define CR_LN_CASE(V)                                                                          \
@@ -360,7 +366,7 @@ cr_status launch_layernorm(const float* x, const float* add, int64_t ld_add, flo
         constexpr int W = (V % 2 == 0) ? 2 : 1;                                                \
         const int grid = static_cast<int>((M + 8 / W - 1) / (8 / W));                          \
         return launch_pdl(layernorm_kernel<V, W>, dim3(grid), dim3(256), 0, st, x, add, ld_add, \
-                          x_out, g, b, eps, M, u);                                             \
+                          x_out, g, b, eps, M, u, x_copy);                                     \
     }
         CR_LN_CASE(1)
         CR_LN_CASE(2)

@@ -5,9 +5,11 @@
 //   rowsq_kernel         per row: the loss head's partial sums of r^2 in order
 //   loss_reduce_kernel   per request, rows summed in order (fp64): the loss
 //   colsum_kernel        column sums in a fixed order (bias, LayerNorm grads)
-//   ln_backward_kernel   LayerNorm backward per row, plus dy * x_hat per element
-//   gelu_backward_kernel dpre = dg * (Phi(pre) + pre phi(pre))
-//   rope_backward_kernel the repairer RoPE's transpose on dQ, dK
+//                        of a signal as it is, through GELU' or through the
+//                        transpose of the repairer RoPE
+//   ln_backward_kernel   LayerNorm backward per row, its bf16 copy and the partial
+//                        column sums of its three parameter gradients
+//   ln_param_kernel      those partial sums in order
 //   sqnorm_*             squared L2 norm of the gradient (fp64, fixed order)
 //   adamw_kernel         clipping coefficient, AdamW, bf16 mirror of the weights
 //   seg_grad_kernel      the segment weights' gradient out of the grouped GEMM's blocks
@@ -111,23 +113,81 @@ __global__ void loss_total_kernel(const double* __restrict__ per_req, int n_req,
 // (eight loads in flight), the warps' sums are added in warp order into
 // partial[y][c], and the last block of column block x to finish (elected by a
 // counter, after a fence) adds the slices in order and resets the counter.
-// The order of the additions never depends on timing.  kOut16: an fp32 input
+// The order of the additions never depends on timing.  kOut16: an fp32 signal
 // is also written rounded to bf16 (round to nearest even) into a16 [rows,
 // cols], the operand of the backward's GEMMs, from the same read.  cols and
-// lda are even.
+// lda are even.  The signal comes from a source: stored values, or dg through
+// GELU', or dQKV through the transposed RoPE, so that these never make a pass of
+// their own (3316 tokens, launch list, cold: GELU' 40 + 19 us as two launches, 46 as one;
+// RoPE 20 + 19 and 32).
 constexpr int kColSlice = 256;
-__device__ __forceinline__ float2 ld2(const float* p, int64_t i) {
-    return *reinterpret_cast<const float2*>(p + i);
-}
-__device__ __forceinline__ float2 ld2(const uint16_t* p, int64_t i) {
-    const uint32_t v = *reinterpret_cast<const uint32_t*>(p + i);
-    return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
-}
-template <typename T, bool kOut16>
+template <typename T>
+struct PlainSrc {
+    static constexpr int kStage = 0;   // float2 of shared memory that stage() fills
+    const T* a;
+    int64_t lda;
+    __device__ __forceinline__ void stage(float2*, int64_t) const {}
+    __device__ __forceinline__ float2 at(int64_t r, int64_t c, const float2*) const {
+        if constexpr (sizeof(T) == 4) {
+            return *reinterpret_cast<const float2*>(a + r * lda + c);
+        } else {
+            const uint32_t v = *reinterpret_cast<const uint32_t*>(a + r * lda + c);
+            return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
+        }
+    }
+};
+// dpre = dg * GELU'(pre), GELU'(x) = Phi(x) + x phi(x)
+struct GeluSrc {
+    static constexpr int kStage = 0;
+    const float *dg, *pre;
+    int64_t lda;
+    __device__ __forceinline__ void stage(float2*, int64_t) const {}
+    static __device__ __forceinline__ float slope(float x) {
+        const float Phi = 0.5f * erfcf(-x * 0.70710678118654752f);
+        const float phi = 0.39894228040143268f * expf(-0.5f * x * x);
+        return fmaf(x, phi, Phi);
+    }
+    __device__ __forceinline__ float2 at(int64_t r, int64_t c, const float2*) const {
+        const float2 x = *reinterpret_cast<const float2*>(pre + r * lda + c);
+        const float2 d = *reinterpret_cast<const float2*>(dg + r * lda + c);
+        return make_float2(d.x * slope(x.x), d.y * slope(x.y));
+    }
+};
+// The repairer RoPE rotated q and k of every head by angle p_t f_i (pairs
+// (i, i + d/2)); its transpose rotates the gradients back:
+//   (a, b) -> (a cos + b sin, b cos - a sin).  dqkv [N, 3 d_b] fp32, Q and K
+// columns [0, 2 d_b); table [d/2, N] (cos, sin) of the forward, angle-major.  A head
+// of d = 32 or 64 lies inside a warp's 64 columns, the pair of a lane's columns in
+// the lane d/4 away (whole warps: 3 d_b is a multiple of 64).  The angles of 32 rows are
+// staged in shared memory, read along the table's rows (a lane per angle straight from
+// the table touches 64 lines per row: 40 us instead of 32).
+struct RopeSrc {
+    static constexpr int kStage = 32 * 33;   // [angle][row], padded
+    const float* dqkv;
+    const float2* table;
+    int64_t n, cols, rot;   // tokens, 3 d_b, 2 d_b
+    int half;               // d / 2
+    __device__ __forceinline__ void stage(float2* t, int64_t r0) const {
+        const int lane = static_cast<int>(threadIdx.x & 31);
+        for (int q = static_cast<int>(threadIdx.x >> 5); q < half; q += 8)
+            if (r0 + lane < n) t[q * 33 + lane] = __ldg(table + q * n + r0 + lane);
+    }
+    __device__ __forceinline__ float2 at(int64_t r, int64_t c, const float2* sm) const {
+        const float2 v = *reinterpret_cast<const float2*>(dqkv + r * cols + c);
+        if (c >= rot) return v;   // the same for all lanes: 2 d_b is a multiple of 64
+        const float2 o = make_float2(__shfl_xor_sync(0xffffffffu, v.x, half / 2),
+                                     __shfl_xor_sync(0xffffffffu, v.y, half / 2));
+        const int j = static_cast<int>(c) & (2 * half - 1), q = j & (half - 1);
+        const float2* t = sm + static_cast<int>(r & 31);
+        const float2 t0 = t[q * 33], t1 = t[(q + 1) * 33];
+        if (j < half) return make_float2(v.x * t0.x + o.x * t0.y, v.y * t1.x + o.y * t1.y);
+        return make_float2(v.x * t0.x - o.x * t0.y, v.y * t1.x - o.y * t1.y);
+    }
+};
+template <typename Src, bool kOut16>
 __global__ void __launch_bounds__(256)
-    colsum_kernel(const T* __restrict__ a, int64_t rows, int64_t cols, int64_t lda,
-                  uint16_t* __restrict__ a16, float* part, float* __restrict__ out, int accumulate,
-                  unsigned* __restrict__ counters) {
+    colsum_kernel(const Src src, int64_t rows, int64_t cols, uint16_t* __restrict__ a16, float* part,
+                  float* __restrict__ out, int accumulate, unsigned* __restrict__ counters) {
     pdl_launch_dependents();
     pdl_wait();
     const int lane = static_cast<int>(threadIdx.x & 31), w = static_cast<int>(threadIdx.x >> 5);
@@ -135,14 +195,28 @@ __global__ void __launch_bounds__(256)
     const int64_t r0 = static_cast<int64_t>(blockIdx.y) * kColSlice;
     const int64_t r1 = min(rows, r0 + kColSlice);
     float s0 = 0.0f, s1 = 0.0f;
-    if (c < cols) {
-#pragma unroll 8
-        for (int64_t r = r0 + w; r < r1; r += 8) {
-            const float2 v = ld2(a, r * lda + c);
-            s0 += v.x;
-            s1 += v.y;
-            if constexpr (kOut16) *reinterpret_cast<uint32_t*>(a16 + r * cols + c) = pack_bf16x2(v.x, v.y);
+    auto row = [&](int64_t r, const float2* sm) {
+        const float2 v = src.at(r, c, sm);
+        s0 += v.x;
+        s1 += v.y;
+        if constexpr (kOut16) *reinterpret_cast<uint32_t*>(a16 + r * cols + c) = pack_bf16x2(v.x, v.y);
+    };
+    if constexpr (Src::kStage > 0) {
+        __shared__ float2 stage[2][Src::kStage];
+        src.stage(stage[0], r0);
+        for (int64_t b = r0; b < r1; b += 32) {   // kColSlice is a multiple of 32
+            const float2* sm = stage[(b >> 5) & 1];
+            __syncthreads();
+            if (b + 32 < r1) src.stage(stage[((b >> 5) & 1) ^ 1], b + 32);
+            if (c < cols) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (b + w + 8 * u < r1) row(b + w + 8 * u, sm);
+            }
         }
+    } else if (c < cols) {
+#pragma unroll 8
+        for (int64_t r = r0 + w; r < r1; r += 8) row(r, nullptr);
     }
     __shared__ float2 red[8][32];
     red[w][lane] = make_float2(s0, s1);
@@ -178,104 +252,124 @@ __global__ void __launch_bounds__(256)
 
 // LayerNorm backward, one warp per row of D (a multiple of 32, at most 1024)
 // values: with x_hat = (x - mean) rstd and g = dy gamma,
-//   dx = rstd (g - mean(g) - x_hat mean(g x_hat))  (+ add, if given)
-// and gprod = dy x_hat per element (its column sums are dgamma).
-__global__ void __launch_bounds__(256)
+//   dx = rstd (g - mean(g) - x_hat mean(g x_hat))  (+ add, if given),
+// also written rounded to bf16 into dx16, the operand of the products that follow.
+// Each lane keeps the column sums of its 32 columns over its rows: dy x_hat (dgamma),
+// dy (dbeta) and dx (the bias gradient of the linear before); a block adds its eight
+// warps' sums in warp order into part [3][blocks][D], ln_param_kernel the blocks' in
+// order.  One pass instead of four: with dy x_hat stored and three column-sum launches
+// after it, each of the thirteen LayerNorms of a 3316-token update took 22 + 2 x 13 + 17
+// us, now 24 + 6 (launch list, cold).
+constexpr int kLnBlocks = 148;
+__host__ __device__ inline int64_t ln_rows_per_block(int64_t n) { return 8 * ((n + 8 * kLnBlocks - 1) / (8 * kLnBlocks)); }
+__global__ void __launch_bounds__(256, 1)
     ln_backward_kernel(const float* __restrict__ x, const float* __restrict__ gamma,
                        const float* __restrict__ dy, const float* __restrict__ add, float eps, int64_t N,
-                       int D, float* __restrict__ dx, float* __restrict__ gprod) {
+                       int D, float* __restrict__ dx, uint16_t* __restrict__ dx16, float* __restrict__ part) {
     pdl_launch_dependents();
     pdl_wait();
-    const int lane = threadIdx.x & 31;
-    const int64_t row = blockIdx.x * static_cast<int64_t>(blockDim.x / 32) + (threadIdx.x >> 5);
-    if (row >= N) return;
-    const float* xr = x + row * D;
-    const float* dr = dy + row * D;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t per_block = ln_rows_per_block(N);
+    const int64_t r0 = blockIdx.x * per_block, r1 = min(N, r0 + per_block);
     const int per = D / 32;   // <= 32
-    float xv[32], gv[32];
+    float ag[32], ab[32], ad[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) ag[i] = ab[i] = ad[i] = 0.0f;
+    for (int64_t row = r0 + w; row < r1; row += 8) {
+        const float* xr = x + row * D;
+        const float* dr = dy + row * D;
+        float xv[32], gv[32];
+        float s = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (i < per) {
+                xv[i] = xr[i * 32 + lane];
+                gv[i] = dr[i * 32 + lane];
+                s += xv[i];
+            }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const float mean = s / D;
+        float v = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (i < per) {
+                const float d = xv[i] - mean;
+                v = fmaf(d, d, v);
+            }
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        const float rstd = rsqrtf(v / D + eps);
+        float sg = 0.0f, sgx = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (i < per) {
+                const float dyv = gv[i];
+                xv[i] = (xv[i] - mean) * rstd;
+                gv[i] = dyv * __ldg(gamma + i * 32 + lane);
+                sg += gv[i];
+                sgx = fmaf(gv[i], xv[i], sgx);
+                ag[i] += dyv * xv[i];
+                ab[i] += dyv;
+            }
+        for (int o = 16; o > 0; o >>= 1) {
+            sg += __shfl_xor_sync(0xffffffffu, sg, o);
+            sgx += __shfl_xor_sync(0xffffffffu, sgx, o);
+        }
+        const float mg = sg / D, mgx = sgx / D;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (i < per) {
+                const int64_t k = row * D + i * 32 + lane;
+                float d = rstd * (gv[i] - mg - xv[i] * mgx);
+                if (add) d += add[k];
+                dx[k] = d;
+                dx16[k] = f32_to_bf16(d);
+                ad[i] += d;
+            }
+    }
+    __shared__ float red[8][1024];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (k) __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (i < per) red[w][i * 32 + lane] = k == 0 ? ag[i] : (k == 1 ? ab[i] : ad[i]);
+        __syncthreads();
+        for (int c = threadIdx.x; c < D; c += 256) {
+            float t = 0.0f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) t += red[u][c];
+            part[(static_cast<int64_t>(k) * gridDim.x + blockIdx.x) * D + c] = t;
+        }
+    }
+}
+
+// Column c of sum k: the blocks' partial sums, warp w of 8 its eighth of the blocks in
+// order, then the warps' in order.
+struct LnParamOut {
+    float* out[3];    // dgamma, dbeta, the column sums of dx
+    float* also;      // a second place for the last (or null)
+};
+__global__ void __launch_bounds__(256)
+    ln_param_kernel(const float* __restrict__ part, int blocks, int D, const LnParamOut o) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int c = blockIdx.x * 32 + lane, k = blockIdx.y;   // D is a multiple of 32
+    const int per = (blocks + 7) / 8;
+    const int b0 = w * per, b1 = min(blocks, b0 + per);
+    const float* p = part + static_cast<int64_t>(k) * blocks * D + c;
     float s = 0.0f;
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) s += p[static_cast<int64_t>(b) * D];
+    __shared__ float red[8][32];
+    red[w][lane] = s;
+    __syncthreads();
+    if (w != 0) return;
+    float t = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 32; ++i)
-        if (i < per) {
-            xv[i] = xr[i * 32 + lane];
-            s += xv[i];
-        }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const float mean = s / D;
-    float v = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 32; ++i)
-        if (i < per) {
-            const float d = xv[i] - mean;
-            v = fmaf(d, d, v);
-        }
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const float rstd = rsqrtf(v / D + eps);
-    float sg = 0.0f, sgx = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 32; ++i)
-        if (i < per) {
-            const int c = i * 32 + lane;
-            const float dyv = dr[c];
-            xv[i] = (xv[i] - mean) * rstd;
-            gv[i] = dyv * __ldg(gamma + c);
-            sg += gv[i];
-            sgx = fmaf(gv[i], xv[i], sgx);
-            gprod[row * D + c] = dyv * xv[i];
-        }
-    for (int o = 16; o > 0; o >>= 1) {
-        sg += __shfl_xor_sync(0xffffffffu, sg, o);
-        sgx += __shfl_xor_sync(0xffffffffu, sgx, o);
-    }
-    const float mg = sg / D, mgx = sgx / D;
-#pragma unroll
-    for (int i = 0; i < 32; ++i)
-        if (i < per) {
-            const int64_t k = row * D + i * 32 + lane;
-            float d = rstd * (gv[i] - mg - xv[i] * mgx);
-            if (add) d += add[k];
-            dx[k] = d;
-        }
-}
-
-// dpre = dg * GELU'(pre), GELU'(x) = Phi(x) + x phi(x), in place on dg.
-__global__ void __launch_bounds__(256)
-    gelu_backward_kernel(float* __restrict__ dg, const float* __restrict__ pre, int64_t n) {
-    pdl_launch_dependents();
-    pdl_wait();
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const float x = pre[i];
-        const float Phi = 0.5f * erfcf(-x * 0.70710678118654752f);
-        const float phi = 0.39894228040143268f * expf(-0.5f * x * x);
-        dg[i] *= fmaf(x, phi, Phi);
-    }
-}
-
-// The repairer RoPE rotated q and k of every head by angle p_t f_i (pairs
-// (i, i + d/2)); its transpose rotates the gradients back:
-//   (a, b) -> (a cos + b sin, b cos - a sin).  dqkv [N, 3 d_b] fp32, Q and K
-// columns [0, 2 d_b); table [d/2, N] (cos, sin) of the forward, angle-major.
-__global__ void __launch_bounds__(256)
-    rope_backward_kernel(float* __restrict__ dqkv, const float2* __restrict__ table, int64_t N, int db,
-                         int hd) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int half = hd / 2;
-    const int64_t pairs_per_row = static_cast<int64_t>(2 * db / hd) * half;   // Q and K heads
-    const int64_t total = N * pairs_per_row;
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t t = i / pairs_per_row;
-        const int64_t rem = i - t * pairs_per_row;
-        const int64_t h = rem / half;
-        const int j = static_cast<int>(rem - h * half);
-        const float2 cs = table[static_cast<int64_t>(j) * N + t];
-        float* base = dqkv + t * 3 * db + h * hd;
-        const float a = base[j], b = base[j + half];
-        base[j] = a * cs.x + b * cs.y;
-        base[j + half] = b * cs.x - a * cs.y;
-    }
+    for (int u = 0; u < 8; ++u) t += red[u][lane];
+    o.out[k][c] = t;
+    if (k == 2 && o.also) o.also[c] = t;
 }
 
 // out[i] = in[i] * scale[i % cols] (dW_seg: the cache's 1 / sigma_stale per column)
@@ -424,43 +518,61 @@ size_t colsum_scratch_floats(int64_t rows, int64_t cols) {
 
 size_t colsum_counters(int64_t cols) { return static_cast<size_t>((cols + 31) / 32); }
 
+namespace {
+template <typename Src, bool kOut16>
+cr_status colsum_launch(const Src& src, int64_t rows, int64_t cols, uint16_t* a16, float* out, bool accumulate,
+                        float* scratch, unsigned* counters, cudaStream_t st) {
+    const int64_t slices = (rows + kColSlice - 1) / kColSlice;
+    if (slices > 65535 || (cols & 1) != 0) return CR_ERR_UNSUPPORTED;
+    const dim3 g1(static_cast<unsigned>((cols + 63) / 64), static_cast<unsigned>(slices));
+    return launch_pdl(colsum_kernel<Src, kOut16>, g1, dim3(256), 0, st, src, rows, cols, a16, scratch, out,
+                      accumulate ? 1 : 0, counters);
+}
+}  // namespace
+
 cr_status launch_colsum_bf16(const float* a, int64_t rows, int64_t cols, uint16_t* a16, float* out,
                              float* scratch, unsigned* counters, cudaStream_t st) {
-    const int64_t slices = (rows + kColSlice - 1) / kColSlice;
-    if (slices > 65535) return CR_ERR_UNSUPPORTED;
-    if ((cols & 1) != 0) return CR_ERR_UNSUPPORTED;
-    const dim3 g1(static_cast<unsigned>((cols + 63) / 64), static_cast<unsigned>(slices));
-    return launch_pdl(colsum_kernel<float, true>, g1, dim3(256), 0, st, a, rows, cols, cols, a16, scratch, out,
-                      0, counters);
+    return colsum_launch<PlainSrc<float>, true>({a, cols}, rows, cols, a16, out, false, scratch, counters, st);
+}
+
+cr_status launch_gelu_backward(const float* dg, const float* pre, int64_t rows, int64_t cols, uint16_t* a16,
+                               float* out, float* scratch, unsigned* counters, cudaStream_t st) {
+    return colsum_launch<GeluSrc, true>({dg, pre, cols}, rows, cols, a16, out, false, scratch, counters, st);
+}
+
+cr_status launch_rope_backward(const float* dqkv, const float2* table, int64_t N, int db, int hd, uint16_t* a16,
+                               float* out, float* scratch, unsigned* counters, cudaStream_t st) {
+    if ((hd != 32 && hd != 64) || db % 64 != 0) return CR_ERR_UNSUPPORTED;
+    return colsum_launch<RopeSrc, true>({dqkv, table, N, 3LL * db, 2LL * db, hd / 2}, N, 3LL * db, a16, out, false,
+                                        scratch, counters, st);
 }
 
 cr_status launch_colsum(const void* a, bool bf16, int64_t rows, int64_t cols, int64_t lda, float* out,
                         bool accumulate, float* scratch, unsigned* counters, cudaStream_t st) {
-    const int64_t slices = (rows + kColSlice - 1) / kColSlice;
-    if (slices > 65535) return CR_ERR_UNSUPPORTED;
-    if ((cols & 1) != 0 || (lda & 1) != 0) return CR_ERR_UNSUPPORTED;
-    const dim3 g1(static_cast<unsigned>((cols + 63) / 64), static_cast<unsigned>(slices));
-    uint16_t* none = nullptr;
-    return bf16 ? launch_pdl(colsum_kernel<uint16_t, false>, g1, dim3(256), 0, st,
-                             static_cast<const uint16_t*>(a), rows, cols, lda, none, scratch, out,
-                             accumulate ? 1 : 0, counters)
-                : launch_pdl(colsum_kernel<float, false>, g1, dim3(256), 0, st, static_cast<const float*>(a),
-                             rows, cols, lda, none, scratch, out, accumulate ? 1 : 0, counters);
+    if ((lda & 1) != 0) return CR_ERR_UNSUPPORTED;
+    return bf16 ? colsum_launch<PlainSrc<uint16_t>, false>({static_cast<const uint16_t*>(a), lda}, rows, cols, nullptr,
+                                                           out, accumulate, scratch, counters, st)
+                : colsum_launch<PlainSrc<float>, false>({static_cast<const float*>(a), lda}, rows, cols, nullptr, out,
+                                                        accumulate, scratch, counters, st);
+}
+
+size_t ln_backward_scratch_floats(int64_t N, int D) {
+    const int64_t per = ln_rows_per_block(N);
+    return static_cast<size_t>(3 * ((N + per - 1) / per) * D);
 }
 
 cr_status launch_ln_backward(const float* x, const float* gamma, const float* dy, const float* add, float eps,
-                             int64_t N, int D, float* dx, float* gprod, cudaStream_t st) {
+                             int64_t N, int D, float* dx, uint16_t* dx16, float* dgamma, float* dbeta, float* dbias,
+                             float* dbias2, float* scratch, cudaStream_t st) {
     if (D % 32 != 0 || D > 1024) return CR_ERR_UNSUPPORTED;
-    return launch_pdl(ln_backward_kernel, dim3(static_cast<unsigned>((N + 7) / 8)), dim3(256), 0, st, x, gamma,
-                      dy, add, eps, N, D, dx, gprod);
-}
-
-cr_status launch_gelu_backward(float* dg, const float* pre, int64_t n, cudaStream_t st) {
-    return launch_pdl(gelu_backward_kernel, grid_for(n), dim3(256), 0, st, dg, pre, n);
-}
-
-cr_status launch_rope_backward(float* dqkv, const float2* table, int64_t N, int db, int hd, cudaStream_t st) {
-    return launch_pdl(rope_backward_kernel, grid_for(N * db), dim3(256), 0, st, dqkv, table, N, db, hd);
+    const int64_t per = ln_rows_per_block(N);
+    const int blocks = static_cast<int>((N + per - 1) / per);
+    cr_status s = launch_pdl(ln_backward_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, st, x, gamma, dy,
+                             add, eps, N, D, dx, dx16, scratch);
+    if (s != CR_OK) return s;
+    const LnParamOut o{{dgamma, dbeta, dbias}, dbias2};
+    return launch_pdl(ln_param_kernel, dim3(static_cast<unsigned>(D / 32), 3), dim3(256), 0, st,
+                      static_cast<const float*>(scratch), blocks, D, o);
 }
 
 cr_status launch_seg_grad(const float* blocks, float* g, int64_t S, int64_t dseg, int64_t dh,

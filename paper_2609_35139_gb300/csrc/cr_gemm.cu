@@ -237,6 +237,38 @@ __device__ __forceinline__ void store16_bf16_global(uint16_t* dst, const float* 
                    pack_bf16x2(v[14], v[15]));
 }
 
+// Columns [col, col + W) of a warp's 32 rows of a staged bf16 tile (rows r0 .. r0 + 31) to
+// the rows' places in global memory: `dst` is the calling lane's row there, from the
+// tile's column 0 (NULL: the row is not written).  W / 8 neighbouring lanes write one row's
+// run of W columns, so a store instruction covers whole 32-byte sectors; the lanes of a
+// quarter warp take rows whose swizzle differs, so their reads hit distinct banks.  The
+// paged head, whose epilogue and not its 8 k-blocks a tile sets the pace (2560 tokens of
+// the 3B shape, R_M): 92.4 us with each thread storing its own row, 32 rows and half
+// sectors an instruction, 86.0 us this way.  The loss head, with twice the k-blocks and
+// half the columns a tile, lost by it (466 -> 509 us at 3316 tokens of the 8B shape) and
+// keeps the direct stores.
+template <int W>
+__device__ __forceinline__ void store_rows_bf16(const uint8_t* tile, int r0, int col, uint16_t* dst) {
+    constexpr int CH = W / 8;       // 16-byte chunks of a row's run
+    constexpr int RP = 32 / CH;     // rows per store instruction
+    static_assert(W == 16 || W == 32, "run of a row");
+    const int lane = static_cast<int>(lane_id());
+    const int sub = lane % CH, q = lane / CH;
+    const int rq = W == 32 ? (q >> 1) + 4 * (q & 1) : 2 * (q & 3) + ((q >> 2) & 1) + 8 * (q >> 3);
+    const int c = col + sub * 8;
+    const uint8_t* src = tile + (c >> 6) * 16384;
+    const int ch = (c & 63) >> 3;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 32; k += RP) {
+        uint16_t* d = reinterpret_cast<uint16_t*>(
+            __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), k + rq));
+        const int r = r0 + k + rq;
+        const uint4 v = *reinterpret_cast<const uint4*>(src + r * 128 + ((ch ^ (r & 7)) << 4));
+        if (d) *reinterpret_cast<uint4*>(d + c) = v;
+    }
+}
+
 // 16 consecutive floats of a shared-memory vector (all lanes read the same
 // addresses: broadcast).
 __device__ __forceinline__ void vec16(const float* v, int col, float* out) {
@@ -847,9 +879,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     }
                 }
                 auto put16 = [&](int col, const float* v) {
-                    if constexpr (Cfg::kPaged) {
-                        if (prow) store16_bf16_global(prow + col, v);
-                    } else if constexpr (Cfg::kLoss) {
+                    if constexpr (Cfg::kLoss) {
                         if (dzrow) {
                             float d[16];
 #pragma unroll
@@ -959,6 +989,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                             put16(ta, ka);
                             put16(tb, kb);
                         }
+                        if constexpr (Cfg::kPaged) {
+                            const int ja = s0 + eg * (dh / 4), jb = ja + dh / 2;
+                            if (dh == 128) {
+                                store_rows_bf16<32>(tile, static_cast<int>(quad * 32), ja, prow);
+                                store_rows_bf16<32>(tile, static_cast<int>(quad * 32), jb, prow);
+                            } else {
+                                store_rows_bf16<16>(tile, static_cast<int>(quad * 32), ja, prow);
+                                store_rows_bf16<16>(tile, static_cast<int>(quad * 32), jb, prow);
+                            }
+                        }
                         for (int b = bx0; b < bx0 + nbx; ++b) done_box(b);
                     }
                 } else {
@@ -992,6 +1032,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                         }
                         put16(c, k);
                       }
+                      if constexpr (Cfg::kPaged)
+                          store_rows_bf16<HALF>(tile, static_cast<int>(quad * 32), bx * Cfg::kBoxCols + eg * HALF,
+                                                prow);
                       done_box(bx);
                     }
                 }

@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(256)
     if (threadIdx.x == 0) counters[blockIdx.x] = 0u;
 }
 
-// LayerNorm backward, one warp per row of D (a multiple of 32, at most 1024)
+// LayerNorm backward, one warp per row of D (a multiple of 64, at most 1024)
 // values: with x_hat = (x - mean) rstd and g = dy gamma,
 //   dx = rstd (g - mean(g) - x_hat mean(g x_hat))  (+ add, if given),
 // also written rounded to bf16 into dx16, the operand of the products that follow.
@@ -259,7 +259,11 @@ __global__ void __launch_bounds__(256)
 // warps' sums in warp order into part [3][blocks][D], ln_param_kernel the blocks' in
 // order.  One pass instead of four: with dy x_hat stored and three column-sum launches
 // after it, each of the thirteen LayerNorms of a 3316-token update took 22 + 2 x 13 + 17
-// us, now 24 + 6 (launch list, cold).
+// us, then 24 + 6 (launch list, cold).  A warp's three rows are a chain of loads and four
+// reductions: `add` is read with the rest instead of after them, and bf16 values go out in
+// pairs (an update of 3316 tokens at the 8B shape 6883 -> 6767 us).  The order of every sum
+// and the fused multiply-add of dx are fixed: six blocks of bf16 operands turn a last-bit
+// change here into 6e-4 of the gradients' norm.
 constexpr int kLnBlocks = 148;
 __host__ __device__ inline int64_t ln_rows_per_block(int64_t n) { return 8 * ((n + 8 * kLnBlocks - 1) / (8 * kLnBlocks)); }
 __global__ void __launch_bounds__(256, 1)
@@ -278,7 +282,7 @@ __global__ void __launch_bounds__(256, 1)
     for (int64_t row = r0 + w; row < r1; row += 8) {
         const float* xr = x + row * D;
         const float* dr = dy + row * D;
-        float xv[32], gv[32];
+        float xv[32], gv[32], av[32];
         float s = 0.0f;
 #pragma unroll
         for (int i = 0; i < 32; ++i)
@@ -287,6 +291,9 @@ __global__ void __launch_bounds__(256, 1)
                 gv[i] = dr[i * 32 + lane];
                 s += xv[i];
             }
+        // (read with the rest, not after the reductions)
+#pragma unroll
+        for (int i = 0; i < 32; ++i) av[i] = (add && i < per) ? add[row * D + i * 32 + lane] : 0.0f;
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         const float mean = s / D;
         float v = 0.0f;
@@ -315,15 +322,23 @@ __global__ void __launch_bounds__(256, 1)
             sgx += __shfl_xor_sync(0xffffffffu, sgx, o);
         }
         const float mg = sg / D, mgx = sgx / D;
+        // bf16 pairs: of columns 32 i and 32 (i + 1) the even lane stores its own and its
+        // neighbour's value of the first, the odd lane of the second
+        const bool odd = lane & 1;
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
-            if (i < per) {
-                const int64_t k = row * D + i * 32 + lane;
-                float d = rstd * (gv[i] - mg - xv[i] * mgx);
-                if (add) d += add[k];
-                dx[k] = d;
-                dx16[k] = f32_to_bf16(d);
-                ad[i] += d;
+        for (int i = 0; i < 32; i += 2)
+            if (i < per) {   // D is a multiple of 64
+                float d[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float q = gv[i + u] - mg - xv[i + u] * mgx;
+                    d[u] = add ? fmaf(rstd, q, av[i + u]) : rstd * q;
+                    dx[row * D + (i + u) * 32 + lane] = d[u];
+                    ad[i + u] += d[u];
+                }
+                const float o = __shfl_xor_sync(0xffffffffu, odd ? d[0] : d[1], 1);
+                *reinterpret_cast<uint32_t*>(dx16 + row * D + (i + (odd ? 1 : 0)) * 32 + (lane & ~1)) =
+                    odd ? pack_bf16x2(o, d[1]) : pack_bf16x2(d[0], o);
             }
     }
     __shared__ float red[8][1024];
@@ -564,7 +579,7 @@ size_t ln_backward_scratch_floats(int64_t N, int D) {
 cr_status launch_ln_backward(const float* x, const float* gamma, const float* dy, const float* add, float eps,
                              int64_t N, int D, float* dx, uint16_t* dx16, float* dgamma, float* dbeta, float* dbias,
                              float* dbias2, float* scratch, cudaStream_t st) {
-    if (D % 32 != 0 || D > 1024) return CR_ERR_UNSUPPORTED;
+    if (D % 64 != 0 || D > 1024) return CR_ERR_UNSUPPORTED;
     const int64_t per = ln_rows_per_block(N);
     const int blocks = static_cast<int>((N + per - 1) / per);
     cr_status s = launch_pdl(ln_backward_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, st, x, gamma, dy,

@@ -174,7 +174,9 @@ static_assert(sizeof(Item) == kDesc * 4, "descriptor size");
 // the ring's tiles in order.  (Under the block-diagonal mask the second tile's rows may
 // start later; their leading key tiles are fully masked and contribute exact zeros.)
 // Tile j of an item is key tile kbase / 128 + j; query tile w needs j in [0, n_w), an
-// empty second tile (past the request's end) none.
+// empty second tile (past the request's end) none.  n_w is never negative: every role
+// counts its ring slots by max(n0, n1), also where the chunk map, which is device memory
+// that no host check sees, ends a tile's keys before the pair's first key tile.
 __device__ __forceinline__ Item make_item(const AttnParams& p, int bid, int sweep) {
     Item d;
     d.bid = bid;
@@ -194,8 +196,10 @@ __device__ __forceinline__ Item make_item(const AttnParams& p, int bid, int swee
     d.rs = p.req_start[a];
     d.len = p.req_start[a + 1] - d.rs;
     d.kbase = key_lo(p, d.rs, d.q0) & ~127;
-    d.n0 = (key_hi(p, d.rs, d.len, min(d.q0 + 127, d.len - 1)) - d.kbase + 127) / 128;
-    d.n1 = d.q0 + 128 < d.len ? (key_hi(p, d.rs, d.len, min(d.q0 + 255, d.len - 1)) - d.kbase + 127) / 128 : 0;
+    d.n0 = max(0, (key_hi(p, d.rs, d.len, min(d.q0 + 127, d.len - 1)) - d.kbase + 127) / 128);
+    d.n1 = d.q0 + 128 < d.len
+               ? max(0, (key_hi(p, d.rs, d.len, min(d.q0 + 255, d.len - 1)) - d.kbase + 127) / 128)
+               : 0;
     return d;
 }
 

@@ -309,13 +309,23 @@ __global__ void __launch_bounds__(kThreads, 1)
             int st = 0;
             uint32_t ph = 0;
             uint32_t it = 0, iq = 0;   // descriptors read, items (the end marks have no Q)
+            // An issuer whose wait gave up releases buffers whose fill it has not seen land:
+            // once any role has given up (its flag is set before such a release, and read
+            // after the release was seen), nothing is filled again.
+            auto may_fill = [&](uint64_t* empty, uint32_t parity, unsigned site) -> bool {
+                const uint32_t a = smem_u32(empty);
+                const bool ready = mbar_test_wait(a, parity);
+                int gone = *wc.abort;
+                if (!ready) gone = mbar_wait_slow(a, parity, wc, site) ? *wc.abort : 1;
+                return __all_sync(0xffffffffu, gone == 0);
+            };
             for (int pass = 0;; ++pass) {
                 Item d;
                 for (; ok && next_item(it, &d); ++it, ++iq) {
                     const int head = d.bid % p.n_heads, n_max = max(d.n0, d.n1);
                     uint64_t* qf = &q_full[iq & 1u];
                     uint8_t* qt = smem + Cfg::kQOff + (iq & 1u) * 2 * Cfg::kTileBytes;
-                    if (!(ok = mbar_wait_warp(&q_empty[iq & 1u], ((iq >> 1) & 1u) ^ 1u, wc, 122))) break;
+                    if (!(ok = may_fill(&q_empty[iq & 1u], ((iq >> 1) & 1u) ^ 1u, 122))) break;
                     if (elect_one()) {
                         mbar_expect_tx(qf, 2 * Cfg::kTileBytes);
                         tma_load_2d(qt, &tmQKV, qf, head * D, d.rs + d.q0);
@@ -323,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     __syncwarp();
                     for (int j = 0; j < n_max; ++j) {
-                        if (!(ok = mbar_wait_warp(&kv_empty[st], ph ^ 1u, wc, 121))) break;
+                        if (!(ok = may_fill(&kv_empty[st], ph ^ 1u, 121))) break;
                         uint8_t* kt = smem + Cfg::kKVOff + st * 2 * Cfg::kTileBytes;
                         if (elect_one()) {
                             mbar_expect_tx(&kv_full[st], 2 * Cfg::kTileBytes);
@@ -343,10 +353,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ++it;   // past the end mark
                 if (!meet(pass)) break;
             }
-            if (!ok) {
-                const uint64_t t0 = globaltimer();
-                while (globaltimer() - t0 < 50000ull) {
-                }
+            // (all roles have met: none gives up after this)
+            if (__any_sync(0xffffffffu, *wc.abort != 0)) {
+                // copies may be under way whose reader has given up: the last fill of each
+                // ring slot (those from st on a lap earlier) and of each Q buffer; a wait for
+                // the phase before the first passes
+                for (int s = 0; s < NS; ++s) mbar_wait_landed(&kv_full[s], s < st ? ph : ph ^ 1u);
+                for (uint32_t b = 0; b < 2; ++b) mbar_wait_landed(&q_full[b], (((iq + 1u - b) >> 1) - 1u) & 1u);
             }
         } else if (warp == 1 || warp == 2) {
             // ---------------------------------------------------- MMA issuers
@@ -475,7 +488,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ++it;
                 if (elect_one()) mma_commit(&drain[w]);
                 __syncwarp();
-                mbar_wait_warp(&drain[w], static_cast<uint32_t>(pass), wc, 227);
+                // (an early exit must not leave an MMA that still writes TMEM)
+                if (!mbar_wait_warp(&drain[w], static_cast<uint32_t>(pass), wc, 227))
+                    mbar_wait_landed(&drain[w], static_cast<uint32_t>(pass));
                 if (!meet(pass)) break;
             }
         } else {
@@ -513,7 +528,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                         clc_try_cancel(clc_answer, clc_full);
                     }
                     __syncwarp();
-                    if (!(ok = mbar_wait_warp(clc_full, asked & 1u, wc, 135))) break;
+                    if (!(ok = mbar_wait_warp(clc_full, asked & 1u, wc, 135))) {
+                        mbar_wait_landed(clc_full, asked & 1u);   // the answer is a copy, too
+                        break;
+                    }
                     ++asked;
                     bid = clc_cancelled_block(clc_answer);
                     fence_async_smem();   // read before the next answer overwrites it

@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
     }
     const uint32_t tmem_base = *tmem_slot;
     const WaitCtx wc{abort_flag, p.status};
+    int filled = 0;   // producer: ring fills
 
     if (warp == 0) {
         // ---------------------------------------------------- TMA producer
@@ -171,10 +172,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
             }
         }
         __syncwarp();
-        bool ok = true;
-        for (int j = 0; j < nw; ++j) {
-            const int st = j % NS;
-            if (!(ok = mbar_wait_warp(&kv_empty[st], (static_cast<uint32_t>(j / NS) & 1u) ^ 1u, wc, 131))) break;
+        for (; filled < nw; ++filled) {
+            const int j = filled, st = j % NS;
+            if (!mbar_wait_warp(&kv_empty[st], (static_cast<uint32_t>(j / NS) & 1u) ^ 1u, wc, 131)) break;
             uint8_t* b = smem + Cfg::kRingOff + st * 2 * Cfg::kTileBytes;
             const int row = rs + (w0 + j) * 128;
             if (elect_one()) {
@@ -188,11 +188,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
                 }
             }
             __syncwarp();
-        }
-        if (!ok) {
-            const uint64_t tw = globaltimer();
-            while (globaltimer() - tw < 50000ull) {
-            }
         }
     } else if (warp == 1) {
         // ---------------------------------------------------- MMA issuer
@@ -259,7 +254,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
         }
         if (elect_one()) mma_commit(drain);
         __syncwarp();
-        mbar_wait_warp(drain, 0, wc, 237);
+        // (an early exit must not leave an MMA that still writes TMEM)
+        if (!mbar_wait_warp(drain, 0, wc, 237)) mbar_wait_landed(drain, 0);
     } else if (warp >= 4) {
         // ---------------------------------------------------- elementwise warps
         const uint32_t quad = warp & 3u;
@@ -435,6 +431,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
         tc_fence_before();
     }
     __syncthreads();
+    // (all roles are through: none gives up after this) copies may be under way whose reader
+    // has given up: the own tiles' and the last fill of each ring slot
+    if (warp == 0 && *wc.abort != 0) {
+        mbar_wait_landed(fix_full, 0);
+        for (int j = max(0, filled - NS); j < filled; ++j)
+            mbar_wait_landed(&kv_full[j % NS], static_cast<uint32_t>(j / NS) & 1u);
+    }
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();

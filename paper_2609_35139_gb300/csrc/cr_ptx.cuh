@@ -15,6 +15,7 @@
 #ifndef CR_WAIT_TIMEOUT_NS
 #define CR_WAIT_TIMEOUT_NS 2000000000ull  // 2 s: far above any legitimate wait
 #endif
+#define CR_LANDING_NS 10000000ull         // 10 ms: for copies and MMAs under way at an early exit
 
 namespace cr {
 
@@ -184,6 +185,16 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, c
                                                unsigned site) {
     const bool ok = mbar_wait(bar, parity, w, site);
     return __all_sync(0xffffffffu, ok);
+}
+
+// Before a CTA ends, whatever the abort flag says: wait for asynchronous work that it has
+// started and that ends by itself (bulk copies into its shared memory, MMAs).  A role that
+// gives up leaves its own wait at once, so the work may still be in flight then.
+__device__ __forceinline__ void mbar_wait_landed(uint64_t* bar, uint32_t parity) {
+    const uint32_t a = smem_u32(bar);
+    const uint64_t t0 = globaltimer();
+    while (!mbar_try_wait(a, parity) && globaltimer() - t0 < CR_LANDING_NS) {
+    }
 }
 
 // ----------------------------------------------------------------- CTA pairs

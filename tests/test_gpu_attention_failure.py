@@ -1,5 +1,6 @@
-"""Attention where something is wrong outside it: a chunk map that no host check sees.
-Nothing here faults or hangs a GPU; every wait in the kernel is bounded."""
+"""Attention where something is wrong outside it: a chunk map that no host check sees, a
+wait of an earlier kernel that gave up.  Nothing here faults or hangs a GPU; every wait in
+the kernel is bounded."""
 import numpy as np
 import pytest
 import torch
@@ -45,3 +46,28 @@ def test_keys_that_end_before_the_first_key_tile(mode, tile):
     for r in range(len(reqs)):
         if r not in bad:
             assert torch.equal(got[cu[r]:cu[r + 1]], want[cu[r]:cu[r + 1]]), f"request {r}"
+
+
+@pytest.mark.parametrize("mode", ["block_causal", "block_diagonal"])
+@pytest.mark.parametrize("hd", [64, 32])
+def test_attention_after_a_wait_gave_up(hd, mode):
+    """A kernel before has given up, so this call's waits may give up, too, at any point:
+    the call ends by itself with its copies landed, and once the status is cleared the
+    same call is right again."""
+    g = np.random.default_rng(hd)
+    nh, reqs = 8, [[int(x) for x in g.integers(100, 400, size=3)] for _ in range(20)]
+    db = nh * hd
+    cend, cstart, _, cu = _maps(reqs)
+    qkv = to_dev(F.f32_to_bf16(g.standard_normal((int(cu[-1]), 3 * db)).astype(np.float32)))
+    want = _call(qkv, db, nh, mode, cend, cstart, cu)
+    assert cr.cr_get_device_status()[0] == cr.CR_OK
+    try:
+        cr.cr_wait_selftest()
+        for _ in range(4):
+            _call(qkv, db, nh, mode, cend, cstart, cu)
+        assert cr.cr_get_device_status()[0] == cr.CR_ERR_TIMEOUT
+    finally:
+        cr.cr_clear_device_status()
+    for _ in range(4):
+        assert torch.equal(_call(qkv, db, nh, mode, cend, cstart, cu), want)
+    assert cr.cr_get_device_status()[0] == cr.CR_OK

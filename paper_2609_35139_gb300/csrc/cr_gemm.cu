@@ -567,11 +567,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 }
             }
         }
-        if (!ok) {  // let copies already in flight land before the CTA exits
-            const uint64_t t0 = globaltimer();
-            while (globaltimer() - t0 < 50000ull) {
-            }
-        }
     } else if (warp == 2) {
         if (epi_load) {
             if (elect_one()) tma_prefetch(&tmC);
@@ -689,11 +684,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                                   epi_full);
                     }
                     __syncwarp();
-                }
-            }
-            if (!ok) {
-                const uint64_t t0 = globaltimer();
-                while (globaltimer() - t0 < 50000ull) {
                 }
             }
         }
@@ -1154,6 +1144,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     else
         __syncthreads();
     if (warp == 1) {
+        settle_in_flight(wc);
         __syncwarp();
         tc_fence_after();
         if constexpr (CG == 2)

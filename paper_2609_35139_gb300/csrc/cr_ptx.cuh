@@ -197,6 +197,15 @@ __device__ __forceinline__ void mbar_wait_landed(uint64_t* bar, uint32_t parity)
     }
 }
 
+// The same where no barrier tells for certain what is under way (a pair's copies count on
+// the even CTA's barriers): after all roles have met, a pause if any of them gave up.
+__device__ __forceinline__ void settle_in_flight(const WaitCtx& w) {
+    if (*w.abort == 0) return;
+    const uint64_t t0 = globaltimer();
+    while (globaltimer() - t0 < 1000000ull) {   // 1 ms
+    }
+}
+
 // ----------------------------------------------------------------- CTA pairs
 // Cluster of two CTAs on two SMs sharing one 256-row MMA (tcgen05 cta_group::2).
 __device__ __forceinline__ uint32_t cluster_ctarank() {

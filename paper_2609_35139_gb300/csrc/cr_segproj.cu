@@ -185,11 +185,6 @@ __global__ void __launch_bounds__(224, 1)
                 }
             }
         }
-        if (!ok) {
-            const uint64_t t0 = globaltimer();
-            while (globaltimer() - t0 < 50000ull) {
-            }
-        }
     } else if (warp == 1) {
         // a K=16 step adds 32 bytes (2 units of 16 B) to a descriptor's start
         const uint64_t da0 = smem_desc(smem_u32(smem), 16, 1024, SWZ_128B);
@@ -368,6 +363,7 @@ __global__ void __launch_bounds__(224, 1)
     }
     __syncthreads();
     if (warp == 1) {
+        settle_in_flight(wc);
         __syncwarp();
         tc_fence_after();
         tmem_dealloc(tmem_base, TMEM_COLS);

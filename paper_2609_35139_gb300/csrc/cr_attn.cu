@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!(ok = mbar_wait_warp(loads_out, it & 1u, wc, 134))) break;
                 ++it;
                 bid = -1;
-                if (*redo_any == 0) {
+                if (!__any_sync(0xffffffffu, *redo_any != 0)) {   // one answer for the warp
                     if (elect_one()) {
                         mbar_expect_tx(clc_full, 16);
                         clc_try_cancel(clc_answer, clc_full);

@@ -53,7 +53,7 @@
 // follows the number of instructions in it (about 5.7 clocks each) and how well its
 // registers hold a whole row.  Hence the fixed reference (the running maximum with its
 // votes, its rescale and the two groups' turn taking cost 2440 clocks a pair), the mask
-// built from one word per 32 keys, the unvoted waits, one pair of row sums, and item
+// built from one word per 32 keys, the unvoted waits, and item
 // fields re-read from shared memory instead of kept.  One block per item cost 8700
 // clocks around its tiles (block start, TMEM, barriers, first loads, last products).
 // Measured, us: 5120 tokens of 10 chunks, 16 heads of 64 | 4102 tokens bidirectional |
@@ -118,21 +118,31 @@ __device__ __forceinline__ void mask_chunk(float (&s)[128], int lo, int hi, floa
         for (int i = 0; i < 32; ++i) s[32 * C + i] = (vis & (1u << i)) ? s[32 * C + i] : neg_inf;
     }
 }
-// 2^(s sc - m) of scores 32 c .. 32 c + 31 as bf16 pairs, added to NR / 2 pairs of
-// running row sums.
-template <int C, int NR>
+// 2^(s sc - m) of scores 32 c .. 32 c + 31 as bf16 pairs, added to the tile's row sums.
+// A tile has eight of them, of 16 terms each, which tile_sum adds up: one sum that runs
+// over the keys of a long row loses its small terms (262144 keys of weight 2^-24.3 under
+// one of 1: half their part of the row sum).
+template <int C>
 __device__ __forceinline__ void exp_chunk(const float (&s)[128], float sc, float m, uint32_t* pk,
-                                          float (&rs)[NR]) {
+                                          float (&rs)[8]) {
 #pragma unroll
     for (int i = 0; i < 32; i += 2) {
         float t0, t1;
         ffma2(t0, t1, s[32 * C + i], s[32 * C + i + 1], sc, sc, -m, -m);
         const float e0 = ex2(t0);
         const float e1 = ex2(t1);
-        const int q = (i >> 1) % (NR / 2);
-        fadd2(rs[2 * q], rs[2 * q + 1], rs[2 * q], rs[2 * q + 1], e0, e1);
+        const int q = (i >> 1) & 3;
+        if (C == 0 && i < 8) {
+            rs[2 * q] = e0;
+            rs[2 * q + 1] = e1;
+        } else {
+            fadd2(rs[2 * q], rs[2 * q + 1], rs[2 * q], rs[2 * q + 1], e0, e1);
+        }
         pk[i >> 1] = pack_bf16x2(e0, e1);
     }
+}
+__device__ __forceinline__ float tile_sum(const float (&rs)[8]) {
+    return ((rs[0] + rs[1]) + (rs[2] + rs[3])) + ((rs[4] + rs[5]) + (rs[6] + rs[7]));
 }
 __device__ __forceinline__ float row_max(const float (&s)[128]) {
     float mx[8];   // independent chains
@@ -609,8 +619,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         // handed over once its store has landed.  P_w is free once PV_w of the tile
         // before has completed: the probe's answer comes in under the second chunk's
         // exponentials.
-        auto put_p = [&](const float (&s)[128], float m_ref, auto& rs, bool pv_waited) {
+        auto put_p = [&](const float (&s)[128], float m_ref, bool pv_waited) {
             uint32_t pk[32];
+            float rs[8];
             exp_chunk<0>(s, sc, m_ref, pk, rs);
             const bool pv = pv_waited || mbar_test_wait_at<kOffPV>(bar, (np & 1u) ^ 1u);
             exp_chunk<1>(s, sc, m_ref, pk + 16, rs);
@@ -622,6 +633,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             exp_chunk<2>(s, sc, m_ref, pk, rs);
             exp_chunk<3>(s, sc, m_ref, pk + 16, rs);
             tmem_st32u(tp + 32, pk);
+            l += tile_sum(rs);
             tmem_wait_st();
             hand_over(At<kOffP1>{});
         };
@@ -659,18 +671,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     m = m_new;
                 }
-                float rs8[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) rs8[q] = 0.0f;
                 // (a row whose keys start in a later tile has m = -inf: its P is 0)
-                put_p(s, (m == NEG_INF) ? 0.0f : m, rs8, true);
-                l += ((rs8[0] + rs8[1]) + (rs8[2] + rs8[3])) + ((rs8[4] + rs8[5]) + (rs8[6] + rs8[7]));
+                put_p(s, (m == NEG_INF) ? 0.0f : m, true);
             }
             wait_last();
         };
         // P and l of every key tile; `known`: m is the row's maximum already
         auto sweep = [&](bool known) {
-            float rs[2] = {0.0f, 0.0f};                // a pair of running sums
+            l = 0.0f;
             int fresh = known ? 0 : 1;                 // tiles before this one may find rows without reference
             for (int j = 0; j < n; ++j) {
                 float s[128];
@@ -684,9 +692,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (__any_sync(0xffffffffu, m == kUnseen)) fresh = j + 2;
                 }
                 hand_over(At<kOffFree>{});
-                put_p(s, m, rs, false);
+                put_p(s, m, false);
             }
-            l = rs[0] + rs[1];
             wait_last();
         };
         // (few values live across the key tiles: the softmax threads' registers are full,

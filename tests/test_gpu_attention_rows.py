@@ -1,0 +1,37 @@
+"""Attention rows at the limits of their sums: many small weights under a large one."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_35139_gb300 import cr
+
+pytestmark = pytest.mark.gpu
+
+
+def _call(qkv, db, nh, n):
+    out = torch.full((n, db), float("nan"), dtype=torch.bfloat16, device="cuda")
+    end = torch.full((n,), n, dtype=torch.int32, device="cuda")
+    cr.cr_masked_attention(qkv, db, nh, "bidirectional", end, torch.zeros_like(end), np.array([0, n], np.int32), out)
+    torch.cuda.synchronize()
+    st, word = cr.cr_get_device_status()
+    assert st == cr.CR_OK, word
+    return out
+
+
+@pytest.mark.parametrize("nh,hd,q0,k0", [(2, 64, 8.0, 16.875), (4, 32, 4.0, 23.875)])
+def test_small_weights_under_a_large_one(nh, hd, q0, k0):
+    """One key of weight 1 with V = 1, 262143 keys of weight e^-16.9 (0.39 of the last bit of
+    1 in fp32) with V = 0: every output is 1 / (1 + the sum of the small weights).  A sum
+    that adds them to the large one by one drops them and is 0.6 % or more too small."""
+    n, db = 262144, nh * hd
+    qkv = torch.zeros((n, 3, nh, hd), dtype=torch.bfloat16, device="cuda")
+    qkv[:, 0, :, 0] = q0
+    qkv[0, 1, :, 0] = k0
+    qkv[0, 2] = 1.0
+    small = (n - 1) * float(np.exp(-q0 * k0 / np.sqrt(hd)))
+    want = 1.0 / (1.0 + small)
+    got = _call(qkv.reshape(n, 3 * db), db, nh, n).double()
+    # half a bf16 step below 1, and 1 % of the small weights' part: a tile's 128 of them come
+    # to 50 last bits of 1, of which each tile's addition may round half a bit
+    bound = 2.0 ** -9 + 0.01 * small
+    assert float((got - want).abs().max()) <= bound, (float(got.min()), float(got.max()), want)

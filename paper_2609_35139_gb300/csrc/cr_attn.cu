@@ -41,10 +41,10 @@
 // key, and it stays there: any m gives the same softmax (it cancels in O / l), P is
 // a floating-point number whose rounding does not depend on its scale, and a row's l
 // is at least 1.  So no later tile needs a row maximum, and O is never rescaled.
-// Only a row whose later scores exceed that first maximum by 2^60 could come near
-// fp32's range; the row sums show it at the end of the item, and the CTA runs such an
-// item again before it ends, with the true row maxima (a sweep of S products only,
-// then the softmax).
+// Only a row whose later scores exceed that first maximum by 2^60, or by less under huge
+// values, could come near fp32's range; the row sums and O show it at the end of the item,
+// and the CTA runs such an item again before it ends, with the true row maxima (a sweep of
+// S products only, then the softmax).
 //
 // What bounds it: with d = 64, a pair of 128 x 128 tiles costs the tensor core 1024
 // clocks and each SM sub-partition's special-function unit 1024 (two tiles'
@@ -730,10 +730,20 @@ __global__ void __launch_bounds__(kThreads, 1)
                     hand_over(At<kOffO>{});
                     const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane);
                     const bool valid = qrow < d->len;
-                    if (!kRunning && __any_sync(0xffffffffu, valid && !(l <= kSumLimit)) && d->sweep == SWEEP_FIRST) {
-                        if (lane == 0) {
-                            redo[it & 3u] = d->bid;
-                            *redo_any = 1;
+                    if constexpr (!kRunning) {
+                        // values of up to 2^127 can overflow O while l is below the limit
+                        float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // stays 0 while every o is finite
+#pragma unroll
+                        for (int c = 0; c < D; c += 2) {
+                            const int q = c & 2;
+                            ffma2(z[q], z[q + 1], o[c], o[c + 1], 0.0f, 0.0f, z[q], z[q + 1]);
+                        }
+                        const bool sound = l <= kSumLimit && (z[0] + z[1]) + (z[2] + z[3]) == 0.0f;
+                        if (__any_sync(0xffffffffu, valid && !sound) && d->sweep == SWEEP_FIRST) {
+                            if (lane == 0) {
+                                redo[it & 3u] = d->bid;
+                                *redo_any = 1;
+                            }
                         }
                     }
                     const float inv = 1.0f / l;

@@ -1,9 +1,13 @@
-"""Attention rows at the limits of their sums: many small weights under a large one."""
+"""Attention rows at the limits of their sums: many small weights under a large one, values
+that leave no room above them."""
 import numpy as np
 import pytest
 import torch
 
+import fixtures as F
+import oracle as O
 from paper_2609_35139_gb300 import cr
+from parity_util import as_f64, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -35,3 +39,28 @@ def test_small_weights_under_a_large_one(nh, hd, q0, k0):
     # to 50 last bits of 1, of which each tile's addition may round half a bit
     bound = 2.0 ** -9 + 0.01 * small
     assert float((got - want).abs().max()) <= bound, (float(got.min()), float(got.max()), want)
+
+
+@pytest.mark.parametrize("step", [0, 20, 50])
+@pytest.mark.parametrize("hd", [64, 32])
+def test_huge_values(hd, step):
+    """Values of 2^100 with scores that outgrow the first key tile by about 2^step: the sums
+    before the division pass fp32's range unless the reference follows, the outputs do not."""
+    g = np.random.default_rng(hd + step)
+    nh, n = 4, 700
+    db = nh * hd
+    x = g.standard_normal((n, 3, db)).astype(np.float32)
+    x[128:, 1] *= max(1.0, step / 3 / np.log2(np.e))
+    x[:, 2] *= 2.0 ** 100
+    qkv = F.f32_to_bf16(x.reshape(n, 3 * db))
+    got, q = as_f64(to_host(_call(to_dev(qkv), db, nh, n))), as_f64(qkv)
+    part = lambda i: q[:, i * db:(i + 1) * db].reshape(n, nh, hd)
+    m = O.attention_mask(np.zeros(n, np.int32), "bidirectional")
+    want = O.masked_attention(part(0), part(1), part(2), m).reshape(n, db)
+    mag = O.masked_attention(part(0), part(1), np.abs(part(2)), m).reshape(n, db)
+    smax = np.abs(np.einsum("ihd,jhd->hij", part(0), part(1))).max() / np.sqrt(hd) * np.log2(np.e)
+    # P and the output rounded to bf16 (2^-9 each, 2x margin), and the fp32 score and its
+    # scaled difference: a few 2^-24 of the largest score in the exponent
+    bound = 2.0 ** -8 * (mag + np.abs(want)) + 2.0 ** -20 * smax * mag
+    assert np.isfinite(got).all()
+    assert float((np.abs(got - want) / bound).max()) <= 1.0

@@ -174,43 +174,40 @@ enum Sweep : int { SWEEP_FIRST = 0, SWEEP_MAX = 1, SWEEP_KNOWN = 2 };
 struct Item {
     int bid;     // < 0: no more items
     int sweep;   // Sweep: the softmax, the row maxima alone, the softmax with them known
-    int q0, rs, len, kbase, n0, n1;
+    int head, q0, rs, len, kbase, n0, n1;
 };
-constexpr int kDesc = 8;
+constexpr int kDesc = 9;
 static_assert(sizeof(Item) == kDesc * 4, "descriptor size");
 
-// Heaviest pairs of each request first.  Both query tiles start at the key tile of the
-// pair's first visible key, kbase = 128 * floor(lo(q0) / 128), so that every role takes
-// the ring's tiles in order.  (Under the block-diagonal mask the second tile's rows may
-// start later; their leading key tiles are fully masked and contribute exact zeros.)
-// Tile j of an item is key tile kbase / 128 + j; query tile w needs j in [0, n_w), an
-// empty second tile (past the request's end) none.  n_w is never negative: every role
-// counts its ring slots by max(n0, n1), also where the chunk map, which is device memory
-// that no host check sees, ends a tile's keys before the pair's first key tile.
-__device__ __forceinline__ Item make_item(const AttnParams& p, int bid, int sweep) {
-    Item d;
-    d.bid = bid;
-    d.sweep = sweep;
-    if (bid < 0) {
-        d.q0 = d.rs = d.len = d.kbase = d.n0 = d.n1 = 0;
-        return d;
-    }
-    const int pair = p.n_items - 1 - bid / p.n_heads;
+// Heaviest pairs of each request first.
+__device__ __forceinline__ void locate_item(const AttnParams& p, int bid, Item& d) {
+    const int order = bid / p.n_heads, pair = p.n_items - 1 - order;
     int a = 0, b = p.n_req - 1;   // the request with tile_prefix[r] <= pair
     while (a < b) {
         const int mid = (a + b + 1) >> 1;
         if (p.tile_prefix[mid] <= pair) a = mid;
         else b = mid - 1;
     }
+    d.bid = bid;
+    d.head = bid - order * p.n_heads;
     d.q0 = (pair - p.tile_prefix[a]) * 256;
     d.rs = p.req_start[a];
     d.len = p.req_start[a + 1] - d.rs;
+}
+// Both query tiles start at the key tile of the pair's first visible key,
+// kbase = 128 * floor(lo(q0) / 128), so that every role takes the ring's tiles in order.
+// (Under the block-diagonal mask the second tile's rows may start later; their leading key
+// tiles are fully masked and contribute exact zeros.)  Tile j of an item is key tile
+// kbase / 128 + j; query tile w needs j in [0, n_w), an empty second tile (past the
+// request's end) none.  n_w is never negative: every role counts its ring slots by
+// max(n0, n1), also where the chunk map, which is device memory that no host check sees,
+// ends a tile's keys before the pair's first key tile.
+__device__ __forceinline__ void count_tiles(const AttnParams& p, Item& d) {
     d.kbase = key_lo(p, d.rs, d.q0) & ~127;
     d.n0 = max(0, (key_hi(p, d.rs, d.len, min(d.q0 + 127, d.len - 1)) - d.kbase + 127) / 128);
     d.n1 = d.q0 + 128 < d.len
                ? max(0, (key_hi(p, d.rs, d.len, min(d.q0 + 255, d.len - 1)) - d.kbase + 127) / 128)
                : 0;
-    return d;
 }
 
 // kRunning: the reference is the running maximum.  P's bf16 rounding depends on the
@@ -282,6 +279,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int k = 0; k < 4; ++k) redo[k] = -1;
         fence_barrier_init();
     }
+    // The CTA's own block, as far as it does not depend on an earlier kernel, before the wait
+    // for that; each role then counts its key tiles by itself.  With item 0 handed from the
+    // scheduler through its slot, after the wait, a call of one round of short items was
+    // slower (us: 60 tokens 5.0 instead of 4.3, 1024 tokens block-diagonal 7.4 instead of
+    // 6.5).  The softmax warps read it from the slot: kept in registers it cost them 1 to 6 %.
+    Item own{};
+    locate_item(p, static_cast<int>(blockIdx.x), own);
+    if (threadIdx.x == 96) {
+        const int* v = reinterpret_cast<const int*>(&own);
+#pragma unroll
+        for (int k = 0; k < kDesc; ++k) desc[k] = v[k];
+    }
     if (warp == 1) tmem_alloc(tmem_slot, 512);
     tc_fence_before();
     __syncthreads();
@@ -299,11 +308,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     // The descriptor of the CTA's it-th item, for the producer and issuer warps; false at
     // the end (or when a role has given up).
     auto next_item = [&](uint32_t it, Item* d) -> bool {
-        if (!mbar_wait_warp(&item_full[it & 1u], (it >> 1) & 1u, wc, 131)) return false;
-        int* v = reinterpret_cast<int*>(d);
+        if (it == 0) {
+            *d = own;
+            count_tiles(p, *d);
+        } else {
+            if (!mbar_wait_warp(&item_full[it & 1u], (it >> 1) & 1u, wc, 131)) return false;
+            int* v = reinterpret_cast<int*>(d);
 #pragma unroll
-        for (int k = 0; k < kDesc; ++k) v[k] = desc[(it & 1u) * kDesc + k];
-        __syncwarp();
+            for (int k = 0; k < kDesc; ++k) v[k] = desc[(it & 1u) * kDesc + k];
+            __syncwarp();
+        }
         if (lane == 0) mbar_arrive(&item_empty[it & 1u]);
         return d->bid >= 0;
     };
@@ -332,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int pass = 0;; ++pass) {
                 Item d;
                 for (; ok && next_item(it, &d); ++it, ++iq) {
-                    const int head = d.bid % p.n_heads, n_max = max(d.n0, d.n1);
+                    const int head = d.head, n_max = max(d.n0, d.n1);
                     uint64_t* qf = &q_full[iq & 1u];
                     uint8_t* qt = smem + Cfg::kQOff + (iq & 1u) * 2 * Cfg::kTileBytes;
                     if (!(ok = may_fill(&q_empty[iq & 1u], ((iq >> 1) & 1u) ^ 1u, 122))) break;
@@ -514,7 +528,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             // by one item, never by two)
             uint32_t asked = 0;   // requests made
             auto publish = [&](uint32_t it, int bid, int sweep) -> bool {
-                const Item d = make_item(p, bid, sweep);
+                Item d{};
+                d.bid = bid;
+                d.sweep = sweep;
+                if (bid >= 0) {
+                    locate_item(p, bid, d);
+                    count_tiles(p, d);
+                }
                 if (!mbar_wait_warp(&item_empty[it & 1u], ((it >> 1) & 1u) ^ 1u, wc, 132)) return false;
                 const int* v = reinterpret_cast<const int*>(&d);
                 if (lane == 0) {
@@ -525,10 +545,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 __syncwarp();
                 return true;
             };
-            int bid = static_cast<int>(blockIdx.x);
+            int bid = -1;
             uint32_t it = 0;
             bool ok = true;
-            while (bid >= 0 && (ok = publish(it, bid, SWEEP_FIRST))) {
+            if (lane == 0) mbar_arrive(&item_full[0]);   // item 0 stands there already
+            do {
                 if (!(ok = mbar_wait_warp(loads_out, it & 1u, wc, 134))) break;
                 ++it;
                 bid = -1;
@@ -547,7 +568,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     fence_async_smem();   // read before the next answer overwrites it
                     __syncwarp();
                 }
-            }
+            } while (bid >= 0 && (ok = publish(it, bid, SWEEP_FIRST)));
             if (ok) ok = publish(it++, -1, SWEEP_FIRST);
             if (meet(0)) {
                 for (int k = 0; k < 4 && ok; ++k) {
@@ -674,7 +695,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 // (a row whose keys start in a later tile has m = -inf: its P is 0)
                 put_p(s, (m == NEG_INF) ? 0.0f : m, true);
             }
-            wait_last();
         };
         // P and l of every key tile; `known`: m is the row's maximum already
         auto sweep = [&](bool known) {
@@ -694,7 +714,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 hand_over(At<kOffFree>{});
                 put_p(s, m, false);
             }
-            wait_last();
         };
         // (few values live across the key tiles: the softmax threads' registers are full,
         // and the item's descriptor stays in its slot until all of them are done with it)
@@ -702,16 +721,29 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int pass = 0;; ++pass) {
             for (bool more = true; more; ++it) {
                 const volatile Item* d = reinterpret_cast<const volatile Item*>(desc + (it & 1u) * kDesc);
-                more = mbar_wait_warp(&item_full[it & 1u], (it >> 1) & 1u, wc, 131) && d->bid >= 0;
-                n = !more ? 0 : (w == 0 ? d->n0 : d->n1);
-                if (n > 0) {
+                more = it == 0 || (mbar_wait_warp(&item_full[it & 1u], (it >> 1) & 1u, wc, 131) && d->bid >= 0);
+                n = 0;
+                if (more) {
                     // visible keys of this row, relative to the first key tile (a row past
                     // the request's end is never stored: no mask; with the running maximum it
                     // shares its warp's votes and sees one key)
-                    const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane), len = d->len;
-                    const int rs = d->rs, kbase = d->kbase;
-                    cend = qrow < len ? key_hi(p, rs, len, qrow) - kbase : (kRunning ? 1 - kbase : 1 << 30);
-                    cbeg = qrow < len ? key_lo(p, rs, qrow) - kbase : (kRunning ? -kbase : 0);
+                    Item o;
+                    o.q0 = d->q0;
+                    o.rs = d->rs;
+                    o.len = d->len;
+                    const int qrow = o.q0 + 128 * w + static_cast<int>(quad * 32 + lane);
+                    const bool in = qrow < o.len;
+                    cend = in ? key_hi(p, o.rs, o.len, qrow) : (kRunning ? 1 : 1 << 30);
+                    cbeg = in ? key_lo(p, o.rs, qrow) : 0;
+                    if (it == 0) {
+                        count_tiles(p, o);
+                        n = w == 0 ? o.n0 : o.n1;
+                    } else {
+                        o.kbase = d->kbase;
+                        n = w == 0 ? d->n0 : d->n1;
+                    }
+                    cend -= o.kbase;
+                    cbeg -= o.kbase;
                 }
                 if (n > 0 && d->sweep == SWEEP_MAX) {
                     sweep_max();
@@ -719,6 +751,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (d->sweep == SWEEP_FIRST) m = kRunning ? NEG_INF : kUnseen;
                     if constexpr (kRunning) sweep_running();
                     else sweep(d->sweep == SWEEP_KNOWN);
+                    // (what does not need O before the wait for it)
+                    const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane);
+                    const bool valid = qrow < d->len;
+                    const int head = d->head;
+                    const int64_t row = d->rs + qrow;
+                    uint4* d4 = reinterpret_cast<uint4*>(p.out + row * p.d_b + head * D);
+                    const float inv = 1.0f / l;
+                    // the row's log-sum-exp for a backward pass: P = 2^(s sc - (m + log2 l))
+                    if (kRunning && valid && p.lse)
+                        p.lse[static_cast<int64_t>(head) * p.req_start[p.n_req] + row] = m + log2f(l);
+                    wait_last();
                     // O_w into registers, so that the next item may overwrite it
                     float o[D];
                     if constexpr (D == 64) {
@@ -728,8 +771,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     tmem_wait_ld();
                     hand_over(At<kOffO>{});
-                    const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane);
-                    const bool valid = qrow < d->len;
+                    if (valid) {
+#pragma unroll
+                        for (int c = 0; c < D; c += 8)
+                            d4[c / 8] = make_uint4(pack_bf16x2(o[c] * inv, o[c + 1] * inv),
+                                                   pack_bf16x2(o[c + 2] * inv, o[c + 3] * inv),
+                                                   pack_bf16x2(o[c + 4] * inv, o[c + 5] * inv),
+                                                   pack_bf16x2(o[c + 6] * inv, o[c + 7] * inv));
+                    }
                     if constexpr (!kRunning) {
                         // values of up to 2^127 can overflow O while l is below the limit
                         float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // stays 0 while every o is finite
@@ -745,21 +794,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 *redo_any = 1;
                             }
                         }
-                    }
-                    const float inv = 1.0f / l;
-                    if (valid) {
-                        const int head = d->bid % p.n_heads;
-                        const int64_t row = d->rs + qrow;
-                        // the row's log-sum-exp for a backward pass: P = 2^(s sc - (m + log2 l))
-                        if (kRunning && p.lse)
-                            p.lse[static_cast<int64_t>(head) * p.req_start[p.n_req] + row] = m + log2f(l);
-                        uint4* d4 = reinterpret_cast<uint4*>(p.out + row * p.d_b + head * D);
-#pragma unroll
-                        for (int c = 0; c < D; c += 8)
-                            d4[c / 8] = make_uint4(pack_bf16x2(o[c] * inv, o[c + 1] * inv),
-                                                   pack_bf16x2(o[c + 2] * inv, o[c + 3] * inv),
-                                                   pack_bf16x2(o[c + 4] * inv, o[c + 5] * inv),
-                                                   pack_bf16x2(o[c + 6] * inv, o[c + 7] * inv));
                     }
                 }
                 __syncwarp();

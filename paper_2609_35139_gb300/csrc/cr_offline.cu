@@ -50,11 +50,10 @@ __device__ __forceinline__ void store8(float* p, const float* v) {
 // assembly before it (3264 tokens of the 8B shape; the rotation reads and writes 0.43
 // GB): 234 us with ranges of layers as neighbouring lanes and two segments in flight,
 // 221 with four in flight, 211 in this order with four, 206 with eight.
-constexpr int kParts = 4;   // layer ranges
 constexpr int kSegs = 8;
 template <typename T>
 __global__ void __launch_bounds__(256) canon_kernel(T* kv, int64_t n, const int32_t* __restrict__ pos,
-                                                    int L, int H, int dh,
+                                                    int L, int H, int dh, int parts_log2,
                                                     const __grid_constant__ Freq f, float dir) {
     pdl_launch_dependents();
     pdl_wait();
@@ -62,13 +61,14 @@ __global__ void __launch_bounds__(256) canon_kernel(T* kv, int64_t n, const int3
     const int lanes = groups * H;   // threads of one (token, layer range)
     const int64_t D = static_cast<int64_t>(2) * L * H * dh;
     const int64_t layer = static_cast<int64_t>(2) * H * dh;
-    const int64_t work = n * lanes * kParts;
+    const int parts = 1 << parts_log2;   // layer ranges
+    const int64_t work = n * lanes * parts;
     for (int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; idx < work;
          idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const int64_t tp = idx / lanes;
         const int gh = static_cast<int>(idx - tp * lanes);
-        const int64_t t = tp / kParts;
-        const int part = static_cast<int>(tp - t * kParts);
+        const int64_t t = tp >> parts_log2;
+        const int part = static_cast<int>(tp) & (parts - 1);
         const int h = gh / groups, g = gh - h * groups;
         const float q = static_cast<float>(__ldg(pos + t));
         float c[8], s[8];
@@ -77,9 +77,9 @@ __global__ void __launch_bounds__(256) canon_kernel(T* kv, int64_t n, const int3
             sincos_prod(q, f.f[g * 8 + i], &s[i], &c[i]);
             s[i] *= dir;
         }
-        const int l1 = (part + 1) * L / kParts;
+        const int l1 = (part + 1) * L / parts;
         T* const first = kv + t * D + h * dh + g * 8;
-        for (int l = part * L / kParts; l < l1; l += kSegs) {
+        for (int l = part * L / parts; l < l1; l += kSegs) {
             float a[kSegs][8], b[kSegs][8];
 #pragma unroll
             for (int u = 0; u < kSegs; ++u) {
@@ -99,6 +99,64 @@ __global__ void __launch_bounds__(256) canon_kernel(T* kv, int64_t n, const int3
                 T* p = first + (l + u) * layer;
                 store8(p, a[u]);
                 store8(p + dh / 2, b[u]);
+            }
+        }
+    }
+}
+
+// The same where the layers are few: a thread's segments run over the heads, too, so that
+// the angles, the larger part of the work there, are worked out once for four segments or
+// so.  Lane p of a token's `step` takes every step-th of its L H segments (layer by layer),
+// from the p-th.  us, by layer ranges / by segments: 20000 tokens of 1 layer of 8 heads 103 /
+// 12, 30000 of 2 layers in fp32 25 / 8, 20000 of 4 layers of 2 heads in fp32 43 / 15; but 128
+// tokens of the last 3.2 / 4.0.  Eight layers as one range instead of four: 24 -> 13 us (3000
+// tokens, 8 heads).
+constexpr int kFew = 4;   // segments in flight
+template <typename T>
+__global__ void __launch_bounds__(256) canon_few_kernel(T* kv, int64_t n, const int32_t* __restrict__ pos,
+                                                        int L, int H, int dh, int step,
+                                                        const __grid_constant__ Freq f, float dir) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int groups = dh / 16;
+    const int lanes = groups * step;
+    const int layer = 2 * H * dh, all = L * H;
+    const int64_t work = n * lanes;
+    for (int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; idx < work;
+         idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int64_t t = idx / lanes;
+        const int gp = static_cast<int>(idx - t * lanes);
+        const int p = gp / groups, g = gp - p * groups;
+        const float q = static_cast<float>(__ldg(pos + t));
+        float c[8], s[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            sincos_prod(q, f.f[g * 8 + i], &s[i], &c[i]);
+            s[i] *= dir;
+        }
+        T* const row = kv + t * L * layer + g * 8;
+        int l = p / H, h = p - l * H;   // the next segment's layer and head
+        for (int k = p; k < all; k += kFew * step) {
+            T* seg[kFew];
+            float a[kFew][8], b[kFew][8];
+#pragma unroll
+            for (int u = 0; u < kFew; ++u) {
+                seg[u] = u == 0 || k + u * step < all ? row + l * layer + h * dh : seg[0];
+                load8(seg[u], a[u]);
+                load8(seg[u] + dh / 2, b[u]);
+                for (h += step; h >= H; h -= H) ++l;
+            }
+#pragma unroll
+            for (int u = 0; u < kFew; ++u) {
+                if (k + u * step >= all) break;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float x = a[u][i], y = b[u][i];
+                    a[u][i] = x * c[i] + y * s[i];
+                    b[u][i] = y * c[i] - x * s[i];
+                }
+                store8(seg[u], a[u]);
+                store8(seg[u] + dh / 2, b[u]);
             }
         }
     }
@@ -196,15 +254,28 @@ cr_status launch_canonicalize(void* kv, bool f32, int64_t n, const int32_t* pos,
     if (dh != 64 && dh != 128) return CR_ERR_UNSUPPORTED;
     Freq f{};
     for (int i = 0; i < dh / 2; ++i) f.f[i] = inv_freq_host[i];
-    const int64_t work = n * (dh / 16) * H * kParts;
-    int64_t blocks = (work + 255) / 256;
-    if (blocks > static_cast<int64_t>(num_sms()) * 16) blocks = static_cast<int64_t>(num_sms()) * 16;
-    const dim3 grid(static_cast<unsigned>(blocks)), block(256);
-    if (f32)
-        return launch_pdl(canon_kernel<float>, grid, block, 0, st, static_cast<float*>(kv), n, pos, L, H,
-                          dh, f, dir);
-    return launch_pdl(canon_kernel<uint16_t>, grid, block, 0, st, static_cast<uint16_t*>(kv), n, pos, L,
-                      H, dh, f, dir);
+    const int groups = dh / 16;
+    const auto grid_of = [](int64_t work) {
+        const int64_t blocks = std::min<int64_t>((work + 255) / 256, static_cast<int64_t>(num_sms()) * 16);
+        return dim3(static_cast<unsigned>(blocks));
+    };
+    // Few layers: threads that share the angles over the heads, once they are two warps an SM
+    // or more.  Fewer (and the angles' cost does not show) take a layer each.
+    const int step = std::max(1, L * H / 4);
+    if (L < kSegs && n * groups * step >= static_cast<int64_t>(num_sms()) * 64) {
+        const dim3 grid = grid_of(n * groups * step);
+        return f32 ? launch_pdl(canon_few_kernel<float>, grid, dim3(256), 0, st, static_cast<float*>(kv), n, pos, L, H,
+                                dh, step, f, dir)
+                   : launch_pdl(canon_few_kernel<uint16_t>, grid, dim3(256), 0, st, static_cast<uint16_t*>(kv), n, pos,
+                                L, H, dh, step, f, dir);
+    }
+    // else ranges of at most eight layers or so a thread, four ranges at most
+    const int parts_log2 = L < kSegs || L >= 20 ? 2 : (L >= 12 ? 1 : 0);
+    const dim3 grid = grid_of((n * groups * H) << parts_log2);
+    return f32 ? launch_pdl(canon_kernel<float>, grid, dim3(256), 0, st, static_cast<float*>(kv), n, pos, L, H, dh,
+                            parts_log2, f, dir)
+               : launch_pdl(canon_kernel<uint16_t>, grid, dim3(256), 0, st, static_cast<uint16_t*>(kv), n, pos, L, H,
+                            dh, parts_log2, f, dir);
 }
 
 cr_status launch_sigma_accumulate(const void* a, const void* b, bool f32, int64_t n, int64_t D,

@@ -1259,30 +1259,42 @@ cr_status launch_gemm(const uint16_t* A, int64_t lda, const uint16_t* W, int64_t
     // ceil(tiles / pairs) rounds.  Pick the instantiated width with the least
     // rounds x (256 + BN) (ties: the wider tile).  The width does not change
     // any output element's K order, so results do not depend on it.
-    // (The fp32 residual add had 160 and 128 only; with 256, O and FC2 of 95617
-    // tokens at N = 512 take 10 rounds instead of 20: the block 1590 -> 1458 us.)
+    // The fp32 residual add picks between 160 and 128 that way, and takes 256 instead for
+    // an A that is walked in bands or where that comes out less at rounds x (64 + BN): its
+    // epilogue, in place on an fp32 tile, grows with BN more than the k-blocks do.  us, 256
+    // against the narrower: 95617 tokens at N = 512, 10 rounds instead of 20, the block 1458 /
+    // 1590; 9000 x 1024, K = 1024, 2 rounds instead of 4, 19.6 / 22.3; but 3000 x 2048,
+    // K = 512, 2 instead of 3, 15.3 / 14.1, and 17000 x 640, K = 640, 3 instead of 4, 21.5 / 20.7.
     int BN;
+    // (an fp32 tile updated in place shares L2 with A: bands from 128 MB of both; us, without
+    // and with: 60000 x 512, K = 512 59.4 / 55.1; 9000 x 4096, K = 1024 71.2 / 66.7)
+    double band_from = 64e6;
+    if (epi == EPI_ADD_F32)
+        band_from = std::min(band_from, std::max(0.0, 128e6 - 4.0 * static_cast<double>(M) * static_cast<double>(N)));
     if (kv) {
         BN = (epi == EPI_KV_F32 || epi == EPI_KV_LOSS) ? 128 : 256;
     } else {
         const int64_t pairs = num_sms() / kCG > 0 ? num_sms() / kCG : 1;
         const int64_t mt = (M + BM * kCG - 1) / (BM * kCG);
-        static const int kF32W[] = {256, 160, 128};
+        static const int kF32W[] = {160, 128};
         static const int kBf16W[] = {256, 192, 128};
         const int* cand = f32_tile ? kF32W : kBf16W;
-        const int nc = 3;
+        const int nc = f32_tile ? 2 : 3;
+        const auto rounds = [&](int w) { return (mt * ((N + w - 1) / w) + pairs - 1) / pairs; };
         BN = cand[0];
         int64_t best = -1;
         for (int i = 0; i < nc; ++i) {
             const int w = cand[i];
             if (epi == EPI_QKV_ROPE && (p.rope_dim <= 0 || w % p.rope_dim != 0)) continue;
-            const int64_t tiles = mt * ((N + w - 1) / w);
-            const int64_t cost = ((tiles + pairs - 1) / pairs) * (256 + w);
+            const int64_t cost = rounds(w) * (256 + w);
             if (best < 0 || cost < best) {
                 best = cost;
                 BN = w;
             }
         }
+        if (f32_tile && (static_cast<double>(M) * static_cast<double>(K) * 2.0 > band_from ||
+                         rounds(256) * (64 + 256) <= rounds(BN) * (64 + BN)))
+            BN = 256;
     }
     if (kv && (N % BN) != 0) return CR_ERR_UNSUPPORTED;
     if (epi == EPI_QKV_ROPE && (BN % p.rope_dim) != 0) return CR_ERR_UNSUPPORTED;
@@ -1303,7 +1315,7 @@ cr_status launch_gemm(const uint16_t* A, int64_t lda, const uint16_t* W, int64_t
     } else {
         p.col_block = 0;
     }
-    p.band_m = band_rows(M, N, K, A_lo ? 2 : 1, p.num_m, p.num_n, 64e6);
+    p.band_m = band_rows(M, N, K, A_lo ? 2 : 1, p.num_m, p.num_n, band_from);
     CUtensorMap ta, tb, tc;
     if (!make_tmap_2d(&ta, A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, K, M, lda * 2, BK, BM,
                       CU_TENSOR_MAP_SWIZZLE_128B))

@@ -611,7 +611,6 @@ cr_status cr_repair_forward_masked(const cr_target_dims* target, const cr_repair
         return s;
     }
     ap->status = status;
-    ap->running = d.f32 ? 1 : 0;   // an fp32 cache would show a changed rounding of P
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // the block-diagonal mask also needs each token's chunk start: once per forward
     if (mask_mode == CR_MASK_BLOCK_DIAGONAL && d.B > 0) {

@@ -101,7 +101,6 @@ constexpr uint32_t kRegsCtl = 48;
 constexpr uint32_t kRegsSoftmax = 224;
 static_assert(kRegsCtl * 128 + 2 * kRegsSoftmax * 128 <= kRegsLaunch * kThreads,
               "register split exceeds the launch allocation");
-constexpr float kRescaleLog2 = 8.0f;   // training: lazy-rescale threshold (log2 units)
 constexpr float kUnseen = -3.0e38f;     // the reference of a row that has seen no key
 constexpr float kSumLimit = 1.152921504606847e18f;   // 2^60: a larger row sum restarts the CTA
 
@@ -210,12 +209,9 @@ __device__ __forceinline__ void count_tiles(const AttnParams& p, Item& d) {
                : 0;
 }
 
-// kRunning: the reference is the running maximum.  P's bf16 rounding depends on the
-// reference, and fp32 results show it: a training step amplifies the change into 2e-3 of
-// its fp32 gradients' norm after six blocks, an fp32 cache moves by 1e-4.  So the training
-// forward, which also writes each row's log-sum-exp for the backward, and the forward of
-// fp32 caches keep the running maximum, and their results stay bit for bit what they were.
-template <int D, bool kRunning>
+// kLse: also write each row's log-sum-exp (for the training step's backward); the
+// inference forward's instantiation has none of that code.
+template <int D, bool kLse>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_kernel(const __grid_constant__ CUtensorMap tmQKV, const __grid_constant__ AttnParams p) {
     using Cfg = AttnCfg<D>;
@@ -303,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // they walk the items to run again.
     auto meet = [&](int pass) -> bool {
         __syncthreads();
-        return !kRunning && pass == 0 && *redo_any != 0;
+        return pass == 0 && *redo_any != 0;
     };
     // The descriptor of the CTA's it-th item, for the producer and issuer warps; false at
     // the end (or when a role has given up).
@@ -636,23 +632,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                 m = fmaxf(m, row_max(s) * sc);
             }
         };
-        // P of one tile (2^(s*sc - m_ref) as bf16 pairs) in two halves of 64 keys, each
+        // P of one tile (2^(s*sc - m) as bf16 pairs) in two halves of 64 keys, each
         // handed over once its store has landed.  P_w is free once PV_w of the tile
         // before has completed: the probe's answer comes in under the second chunk's
         // exponentials.
-        auto put_p = [&](const float (&s)[128], float m_ref, bool pv_waited) {
+        auto put_p = [&](const float (&s)[128]) {
             uint32_t pk[32];
             float rs[8];
-            exp_chunk<0>(s, sc, m_ref, pk, rs);
-            const bool pv = pv_waited || mbar_test_wait_at<kOffPV>(bar, (np & 1u) ^ 1u);
-            exp_chunk<1>(s, sc, m_ref, pk + 16, rs);
-            if (!pv_waited) settle(pv, kOffPV, (np & 1u) ^ 1u, 322);
+            exp_chunk<0>(s, sc, m, pk, rs);
+            const bool pv = mbar_test_wait_at<kOffPV>(bar, (np & 1u) ^ 1u);
+            exp_chunk<1>(s, sc, m, pk + 16, rs);
+            settle(pv, kOffPV, (np & 1u) ^ 1u, 322);
             ++np;
             tmem_st32u(tp, pk);
             tmem_wait_st();
             hand_over(At<kOffP0>{});
-            exp_chunk<2>(s, sc, m_ref, pk, rs);
-            exp_chunk<3>(s, sc, m_ref, pk + 16, rs);
+            exp_chunk<2>(s, sc, m, pk, rs);
+            exp_chunk<3>(s, sc, m, pk + 16, rs);
             tmem_st32u(tp + 32, pk);
             l += tile_sum(rs);
             tmem_wait_st();
@@ -661,40 +657,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         // the last PV product of an item
         auto wait_last = [&]() {
             settle(mbar_test_wait_at<kOffPV>(bar, (np & 1u) ^ 1u), kOffPV, (np & 1u) ^ 1u, 324);
-        };
-        // the kRunning form: m is the row's running maximum, moved lazily, only
-        // when a tile raises it by more than 2^8 somewhere in the warp (O_w and l are
-        // then rescaled)
-        auto sweep_running = [&]() {
-            l = 0.0f;
-            for (int j = 0; j < n; ++j) {
-                float s[128];
-                take_s(s);
-                mask_s(s, j);
-                hand_over(At<kOffFree>{});
-                const float mx = row_max(s) * sc;
-                wait_last();   // O_w and P_w are free
-                const bool raise = (j == 0) || (mx > m + kRescaleLog2);
-                if (__any_sync(0xffffffffu, raise)) {
-                    const float m_new = fmaxf(m, mx);
-                    if (j > 0) {
-                        const float alpha = (m == m_new) ? 1.0f : ex2(m - m_new);
-#pragma unroll
-                        for (int c = 0; c < D; c += 16) {
-                            float o[16];
-                            tmem_ld16(to + c, o);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) o[i] *= alpha;
-                            tmem_st16(to + c, o);
-                        }
-                        l *= alpha;
-                    }
-                    m = m_new;
-                }
-                // (a row whose keys start in a later tile has m = -inf: its P is 0)
-                put_p(s, (m == NEG_INF) ? 0.0f : m, true);
-            }
         };
         // P and l of every key tile; `known`: m is the row's maximum already
         auto sweep = [&](bool known) {
@@ -712,7 +674,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (__any_sync(0xffffffffu, m == kUnseen)) fresh = j + 2;
                 }
                 hand_over(At<kOffFree>{});
-                put_p(s, m, false);
+                put_p(s);
             }
         };
         // (few values live across the key tiles: the softmax threads' registers are full,
@@ -725,15 +687,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                 n = 0;
                 if (more) {
                     // visible keys of this row, relative to the first key tile (a row past
-                    // the request's end is never stored: no mask; with the running maximum it
-                    // shares its warp's votes and sees one key)
+                    // the request's end is never stored: no mask)
                     Item o;
                     o.q0 = d->q0;
                     o.rs = d->rs;
                     o.len = d->len;
                     const int qrow = o.q0 + 128 * w + static_cast<int>(quad * 32 + lane);
                     const bool in = qrow < o.len;
-                    cend = in ? key_hi(p, o.rs, o.len, qrow) : (kRunning ? 1 : 1 << 30);
+                    cend = in ? key_hi(p, o.rs, o.len, qrow) : 1 << 30;
                     cbeg = in ? key_lo(p, o.rs, qrow) : 0;
                     if (it == 0) {
                         count_tiles(p, o);
@@ -748,9 +709,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (n > 0 && d->sweep == SWEEP_MAX) {
                     sweep_max();
                 } else if (n > 0) {
-                    if (d->sweep == SWEEP_FIRST) m = kRunning ? NEG_INF : kUnseen;
-                    if constexpr (kRunning) sweep_running();
-                    else sweep(d->sweep == SWEEP_KNOWN);
+                    if (d->sweep == SWEEP_FIRST) m = kUnseen;
+                    sweep(d->sweep == SWEEP_KNOWN);
                     // (what does not need O before the wait for it)
                     const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane);
                     const bool valid = qrow < d->len;
@@ -759,7 +719,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     uint4* d4 = reinterpret_cast<uint4*>(p.out + row * p.d_b + head * D);
                     const float inv = 1.0f / l;
                     // the row's log-sum-exp for a backward pass: P = 2^(s sc - (m + log2 l))
-                    if (kRunning && valid && p.lse)
+                    if (kLse && valid)
                         p.lse[static_cast<int64_t>(head) * p.req_start[p.n_req] + row] = m + log2f(l);
                     wait_last();
                     // O_w into registers, so that the next item may overwrite it
@@ -779,20 +739,18 @@ __global__ void __launch_bounds__(kThreads, 1)
                                                    pack_bf16x2(o[c + 4] * inv, o[c + 5] * inv),
                                                    pack_bf16x2(o[c + 6] * inv, o[c + 7] * inv));
                     }
-                    if constexpr (!kRunning) {
-                        // values of up to 2^127 can overflow O while l is below the limit
-                        float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // stays 0 while every o is finite
+                    // values of up to 2^127 can overflow O while l is below the limit
+                    float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // stays 0 while every o is finite
 #pragma unroll
-                        for (int c = 0; c < D; c += 2) {
-                            const int q = c & 2;
-                            ffma2(z[q], z[q + 1], o[c], o[c + 1], 0.0f, 0.0f, z[q], z[q + 1]);
-                        }
-                        const bool sound = l <= kSumLimit && (z[0] + z[1]) + (z[2] + z[3]) == 0.0f;
-                        if (__any_sync(0xffffffffu, valid && !sound) && d->sweep == SWEEP_FIRST) {
-                            if (lane == 0) {
-                                redo[it & 3u] = d->bid;
-                                *redo_any = 1;
-                            }
+                    for (int c = 0; c < D; c += 2) {
+                        const int q = c & 2;
+                        ffma2(z[q], z[q + 1], o[c], o[c + 1], 0.0f, 0.0f, z[q], z[q + 1]);
+                    }
+                    const bool sound = l <= kSumLimit && (z[0] + z[1]) + (z[2] + z[3]) == 0.0f;
+                    if (__any_sync(0xffffffffu, valid && !sound) && d->sweep == SWEEP_FIRST) {
+                        if (lane == 0) {
+                            redo[it & 3u] = d->bid;
+                            *redo_any = 1;
                         }
                     }
                 }
@@ -810,10 +768,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-template <int D, bool kRunning>
+template <int D, bool kLse>
 cr_status launch_d(const CUtensorMap& tm, const AttnParams& p, cudaStream_t st) {
     using Cfg = AttnCfg<D>;
-    auto kern = attn_kernel<D, kRunning>;
+    auto kern = attn_kernel<D, kLse>;
     static unsigned long long attr_done = 0;   // one per template instantiation
     const cr_status sa = ensure_smem_attr(kern, static_cast<int>(Cfg::kSmemBytes), &attr_done);
     if (sa != CR_OK) return sa;
@@ -883,7 +841,7 @@ cr_status launch_attention(const uint16_t* qkv, int64_t n_tokens, int head_dim,
                       3ull * p.d_b * 2, head_dim, 128,
                       head_dim == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
         return CR_ERR_INVALID_ARG;
-    if (p.lse || p.running) return head_dim == 64 ? launch_d<64, true>(tm, p, st) : launch_d<32, true>(tm, p, st);
+    if (p.lse) return head_dim == 64 ? launch_d<64, true>(tm, p, st) : launch_d<32, true>(tm, p, st);
     return head_dim == 64 ? launch_d<64, false>(tm, p, st) : launch_d<32, false>(tm, p, st);
 }
 

@@ -199,7 +199,6 @@ struct AttnParams {
     int32_t req_start[kMaxReq + 1];   // cu_seqlens
     int32_t tile_prefix[kMaxReq + 1]; // cumulative items per request
     float* lse;                  // [heads][N] or null: log2-unit log-sum-exp of each row (training)
-    int32_t running;             // keep the running maximum as softmax reference (set with lse, too)
 };
 
 // attention backward (training step)

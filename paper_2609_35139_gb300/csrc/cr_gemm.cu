@@ -1211,7 +1211,8 @@ cr_status launch_inst(const CUtensorMap& ta, const CUtensorMap& tb, const CUtens
     return cuda_check(cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, p));
 }
 
-// (bands: 256-wide tiles only, the width a launch of that many rows gets)
+// (bands: 256-wide tiles only; a launch whose rule picks a narrower width, as N = 384 or 128
+// do, walks in one band)
 template <int BN, int EPI, int CG, int LAY = LAY_KK>
 cr_status launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc,
                     const GemmParams& p, cudaStream_t st) {

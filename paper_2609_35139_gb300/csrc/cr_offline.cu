@@ -162,14 +162,16 @@ __global__ void __launch_bounds__(256) canon_few_kernel(T* kv, int64_t n, const 
     }
 }
 
-// Partial sums of squares: block (x, y) covers 1024 coordinates (8 per thread)
+// Partial sums of squares: block (x, y) covers 8 THREADS coordinates (8 per thread)
 // over the 64-token slice y; part[y][j].  With b, the squares of a - b.  HBM-bound:
-// blocks of 128 threads leave less of the chip idle in the last round than 256 (4096
-// tokens of the 7B shape against another cache, 0.47 GB: the statistic 107 -> 92 us).
-constexpr int kSigmaThreads = 128;
-template <typename T>
-__global__ void __launch_bounds__(kSigmaThreads) sigma_partial_kernel(const T* __restrict__ a, const T* __restrict__ b,
-                                                            int64_t n, int64_t D, float* __restrict__ part) {
+// blocks of 128 threads leave less of the chip idle in the last round than 256 (5120
+// tokens of the 7B shape against another cache, 0.59 GB: the statistic 142 -> 132 us),
+// but two bf16 caches with rows of 128 KB or more stream unevenly in them at some lengths, and
+// take 192 (the 8B shape, us, 256 / 128 / 192 threads: 4096 tokens 208 / 198 / 202, 5120
+// 242 / 274 / 235, 7000 330 / 366 / 324, 12000 566 / 622 / 556).
+template <typename T, int THREADS>
+__global__ void __launch_bounds__(THREADS) sigma_partial_kernel(const T* __restrict__ a, const T* __restrict__ b,
+                                                                int64_t n, int64_t D, float* __restrict__ part) {
     pdl_launch_dependents();
     pdl_wait();
     const int64_t col = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) * 8;
@@ -282,14 +284,18 @@ cr_status launch_sigma_accumulate(const void* a, const void* b, bool f32, int64_
                                   float* part, double* sumsq, cudaStream_t st) {
     if (n <= 0) return CR_OK;
     const int64_t slices = (n + kSigmaSlice - 1) / kSigmaSlice;
-    const dim3 grid(static_cast<unsigned>((D / 8 + kSigmaThreads - 1) / kSigmaThreads), static_cast<unsigned>(slices));
+    // (in shorter calls, below 2048 tokens of the 8B shape, latency counts and 128 are faster)
+    const bool wide = b && !f32 && D >= 65536 && n * D >= (1 << 27);
+    const int threads = wide ? 192 : 128;
+    const dim3 grid(static_cast<unsigned>((D / 8 + threads - 1) / threads), static_cast<unsigned>(slices));
     cr_status s;
     if (f32)
-        s = launch_pdl(sigma_partial_kernel<float>, grid, dim3(kSigmaThreads), 0, st, static_cast<const float*>(a),
+        s = launch_pdl(sigma_partial_kernel<float, 128>, grid, dim3(threads), 0, st, static_cast<const float*>(a),
                        static_cast<const float*>(b), n, D, part);
     else
-        s = launch_pdl(sigma_partial_kernel<uint16_t>, grid, dim3(kSigmaThreads), 0, st,
-                       static_cast<const uint16_t*>(a), static_cast<const uint16_t*>(b), n, D, part);
+        s = launch_pdl(wide ? sigma_partial_kernel<uint16_t, 192> : sigma_partial_kernel<uint16_t, 128>, grid,
+                       dim3(threads), 0, st, static_cast<const uint16_t*>(a), static_cast<const uint16_t*>(b), n, D,
+                       part);
     if (s != CR_OK) return s;
     const int64_t blocks = (D + 63) / 64;
     return launch_pdl(sigma_reduce_kernel, dim3(static_cast<unsigned>(blocks)), dim3(64), 0, st,

@@ -1226,18 +1226,22 @@ cr_status launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensor
 // A) and a W of N x K.  W-tile-major order walks every row of A for each column tile, which
 // is free while A stays in L2 but reads a larger A from HBM once per column tile (FC2 of
 // 95617 tokens: 392 MB four times).  In bands A is read once and W once per band: one row
-// tile for a W of up to 10 MB, else about 20 MB of A.  0: A below `from` bytes, one band:
+// tile for a W of up to 10 MB, else about band_bytes of A.  0: A below `from` bytes, one band:
 // 64 MB, and for two products in one launch, whose tiles of unequal length are dealt out
 // in few rounds, the 128 MB of L2 (6914 tokens, 99 MB: 300 us in one band, 311 in bands).
 // Measured, us, one band / 40 MB / 20 MB / one row tile: one block of 95617 tokens at
 // d_b = 512 1458 / 1381 / 1375 / 1370; of 71889 tokens at 1024 2573 / 2237 / 2235 / 2184;
 // the 134 MB head of 48033 tokens 4187 / 4296 / 4135 / 4901; its front (W_map 16 MB)
-// 2445 / 2308 / 2226 / 2425.
-int32_t band_rows(int64_t M, int64_t N, int64_t K, int terms, int32_t num_m, int32_t num_n, double from) {
+// 2445 / 2308 / 2226 / 2425.  Heads without R_M take 14 MB: at K = 512, 20 MB are 76 row
+// tiles, one round of the pairs, which then stream the same columns of all their rows in
+// step; R_M spreads them (one band / 14 / 20 MB: 63000 tokens of the 3B shape 1104 / 1102 /
+// 1310, with R_M 1570 / 1380 / 1336; 33000 of the 8B shape 2880 / 2693 / 2754).
+int32_t band_rows(int64_t M, int64_t N, int64_t K, int terms, int32_t num_m, int32_t num_n, double from,
+                  double band_bytes = 20e6) {
     const double row_tile = 256.0 * static_cast<double>(K) * 2.0 * terms;
     if (num_n < 2 || static_cast<double>(M) * static_cast<double>(K) * 2.0 * terms <= from) return 0;
     if (static_cast<double>(N) * static_cast<double>(K) * 2.0 <= 10e6) return 1;
-    const int32_t band = static_cast<int32_t>(20e6 / row_tile);
+    const int32_t band = static_cast<int32_t>(band_bytes / row_tile);
     return band < 1 ? 1 : (band >= num_m ? 0 : band);
 }
 
@@ -1316,7 +1320,7 @@ cr_status launch_gemm(const uint16_t* A, int64_t lda, const uint16_t* W, int64_t
     } else {
         p.col_block = 0;
     }
-    p.band_m = band_rows(M, N, K, A_lo ? 2 : 1, p.num_m, p.num_n, band_from);
+    p.band_m = band_rows(M, N, K, A_lo ? 2 : 1, p.num_m, p.num_n, band_from, kv && !p.rope_on ? 14e6 : 20e6);
     CUtensorMap ta, tb, tc;
     if (!make_tmap_2d(&ta, A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, K, M, lda * 2, BK, BM,
                       CU_TENSOR_MAP_SWIZZLE_128B))

@@ -15,7 +15,9 @@
 // A work item is a (request, head, pair of consecutive 128-query tiles w = 0, 1).  A
 // CTA runs one item after another: its own block's, then items of blocks that have not
 // started, which it takes over by cluster launch control as soon as an item's loads are
-// out, so that the next item's Q, K and V arrive under this one's last tiles.  Three
+// out, so that the next item's Q, K and V arrive under this one's last tiles.  The item
+// scheduler hands those on through two slots of shared memory; the own one is located
+// before the wait for the kernel before, and nothing waits for the scheduler there.  Three
 // warpgroups, the first of which gives registers to the other two:
 //   warp 0      TMA: both Q tiles of an item (two buffers), then K_j and V_j per key
 //               tile into a 4-deep ring shared by the two query tiles
@@ -38,9 +40,10 @@
 // columns).  The two groups overlap each other's exponentials with their MMAs.
 //
 // The reference m of a row is the maximum of the first key tile in which it sees a
-// key, and it stays there: any m gives the same softmax (it cancels in O / l), P is
-// a floating-point number whose rounding does not depend on its scale, and a row's l
-// is at least 1.  So no later tile needs a row maximum, and O is never rescaled.
+// key, and it stays there: any m gives the same softmax (it cancels in O / l), bf16 rounds
+// P with the same relative error at any scale, and a row's l is at least 1.  So no later
+// tile needs a row maximum, and O is never rescaled.  (Where the scores do not outgrow the
+// first tile's by 2^8, a running maximum moved from 2^8 on gives the same bits.)
 // Only a row whose later scores exceed that first maximum by 2^60, or by less under huge
 // values, could come near fp32's range; the row sums and O show it at the end of the item,
 // and the CTA runs such an item again before it ends, with the true row maxima (a sweep of
@@ -53,14 +56,15 @@
 // follows the number of instructions in it (about 5.7 clocks each) and how well its
 // registers hold a whole row.  Hence the fixed reference (the running maximum with its
 // votes, its rescale and the two groups' turn taking cost 2440 clocks a pair), the mask
-// built from one word per 32 keys, the unvoted waits, and item
-// fields re-read from shared memory instead of kept.  One block per item cost 8700
-// clocks around its tiles (block start, TMEM, barriers, first loads, last products).
+// built from one word per 32 keys, the unvoted waits, and item fields re-read from shared
+// memory instead of kept.  One block per item cost 8700 clocks around its tiles (block
+// start, TMEM, barriers, first loads, last products).
 // Measured, us: 5120 tokens of 10 chunks, 16 heads of 64 | 4102 tokens bidirectional |
 // 5120 tokens block-diagonal | 16 ragged requests of 95617 tokens, 8 heads:
 //   running maximum, a block per item   64.0 | 81.6 | 25.1 | 836
-//   fixed reference                     54.6 | 66.3 | 24.1 | 658
+//   fixed reference, one pair of sums   54.6 | 66.3 | 24.1 | 658
 //   and items taken over                52.4 | 66.1 | 21.1 | 598
+//   as built: eight row sums a tile     52.6 | 66.8 | 21.1 | 601
 // Tried and slower: four softmax warpgroups of half rows (76 us on the second shape:
 // more barrier work and MIO queueing), the next tile's chunks loaded under the last
 // exponentials (89 us), one hand-over of P instead of two halves (+4 %), spinning waits.
@@ -89,7 +93,7 @@ struct AttnCfg {
     static constexpr uint32_t kTmemP = 384;    // P_w at 384 + w * 64 (bf16 pairs)
 };
 
-// Three warpgroups: control (TMA, two MMA issuers, one idle warp) and two
+// Three warpgroups: control (TMA, two MMA issuers, the item scheduler) and two
 // softmax groups.
 // At launch each thread gets 65536 / 384 = 168 registers (the host checks
 // this); the control warpgroup gives up most of its share so that the softmax
@@ -102,7 +106,7 @@ constexpr uint32_t kRegsSoftmax = 224;
 static_assert(kRegsCtl * 128 + 2 * kRegsSoftmax * 128 <= kRegsLaunch * kThreads,
               "register split exceeds the launch allocation");
 constexpr float kUnseen = -3.0e38f;     // the reference of a row that has seen no key
-constexpr float kSumLimit = 1.152921504606847e18f;   // 2^60: a larger row sum restarts the CTA
+constexpr float kSumLimit = 1.152921504606847e18f;   // 2^60: above it the item runs again
 
 // Scores 32 c .. 32 c + 31 of a row whose visible keys, relative to the tile, are
 // [lo, hi): the others become -inf (a fully visible chunk is left alone).
@@ -240,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                           //     softmax warps are done with the item
     uint64_t* loads_out = item_empty + 2; // the loads of an item have all been issued
     uint64_t* clc_full = loads_out + 1;   // the answer to a request for another item
-    // (34 barriers: 272 bytes)
+    // (32 barriers: 256 bytes)
     uint4* clc_answer = reinterpret_cast<uint4*>(smem + Cfg::kBarOff + 320);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + Cfg::kBarOff + 336);
     int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);

@@ -32,8 +32,8 @@ __device__ __forceinline__ uint64_t globaltimer() {
 // The warp index, by a shuffle: the compiler then knows that it is the same in the whole
 // warp, so that branches on the role and addresses made from it stay in uniform registers.
 // Without it every TMEM load, store and MMA address went through a register move first:
-// the pool head with R_M on 3775 ragged rows 193 -> 173 us, the encoder front of 6914
-// tokens 305 -> 297 us.
+// the pool head with R_M on 3775 ragged rows 203 -> 188 us, the encoder front of 6914
+// tokens 307 -> 300 us.
 __device__ __forceinline__ uint32_t warp_id() { return __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0); }
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
 

@@ -39,32 +39,28 @@
 // the PV MMA reads it as the A operand (TMEM holds S_0, S_1, O_0, O_1, P_0, P_1: 512
 // columns).  The two groups overlap each other's exponentials with their MMAs.
 //
-// The reference m of a row is the maximum of the first key tile in which it sees a
-// key, and it stays there: any m gives the same softmax (it cancels in O / l), bf16 rounds
-// P with the same relative error at any scale, and a row's l is at least 1.  So no later
-// tile needs a row maximum, and O is never rescaled.  (Where the scores do not outgrow the
-// first tile's by 2^8, a running maximum moved from 2^8 on gives the same bits.)
-// Only a row whose later scores exceed that first maximum by 2^60, or by less under huge
-// values, could come near fp32's range; the row sums and O show it at the end of the item,
-// and the CTA runs such an item again before it ends, with the true row maxima (a sweep of
-// S products only, then the softmax).
+// The reference m of a row is its running maximum, moved lazily: only where a tile outgrows
+// it by more than 2^8 in some row of the warp does the warp wait for the last product and
+// rescale its O rows in TMEM and its row sums.  Any m gives the same softmax (it cancels in
+// O / l), but not the same rounding of P to bf16: a row's largest P is 1 and exact, which
+// is what counts where one key takes most of the weight.  With the maximum of the first
+// visible key tile as a fixed reference the kernel was 9 % faster and up to 35 % less exact
+// there (scores of 12 times unit variance, relative error 1.7e-3 -> 2.2e-3).
 //
 // What bounds it: with d = 64, a pair of 128 x 128 tiles costs the tensor core 1024
 // clocks and each SM sub-partition's special-function unit 1024 (two tiles'
 // exponentials at 8 a clock; 1126 measured with the packing and the sums), but only
 // two softmax warps share a sub-partition and each is one serial chain, so the time
 // follows the number of instructions in it (about 5.7 clocks each) and how well its
-// registers hold a whole row.  Hence the fixed reference (the running maximum with its
-// votes, its rescale and the two groups' turn taking cost 2440 clocks a pair), the mask
-// built from one word per 32 keys, the unvoted waits, and item fields re-read from shared
-// memory instead of kept.  One block per item cost 8700 clocks around its tiles (block
-// start, TMEM, barriers, first loads, last products).
+// registers hold a whole row.  Hence the mask built from one word per 32 keys, the unvoted
+// waits, no wait for the last product before the exponentials unless O is rescaled, item
+// fields re-read from shared memory instead of kept, and the rescale as a loop (unrolled, its
+// code cost the short calls 0.1 us in instruction fetches).  One block per item cost 8700
+// clocks around its tiles (block start, TMEM, barriers, first loads, last products).
 // Measured, us: 5120 tokens of 10 chunks, 16 heads of 64 | 4102 tokens bidirectional |
 // 5120 tokens block-diagonal | 16 ragged requests of 95617 tokens, 8 heads:
-//   running maximum, a block per item   64.0 | 81.6 | 25.1 | 836
-//   fixed reference, one pair of sums   54.6 | 66.3 | 24.1 | 658
-//   and items taken over                52.4 | 66.1 | 21.1 | 598
-//   as built: eight row sums a tile     52.6 | 66.8 | 21.1 | 601
+//   a block per item, groups in turns   64.2 | 81.8 | 25.3 | 836
+//   as built                            56.9 | 73.3 | 21.5 | 669
 // Tried and slower: four softmax warpgroups of half rows (76 us on the second shape:
 // more barrier work and MIO queueing), the next tile's chunks loaded under the last
 // exponentials (89 us), one hand-over of P instead of two halves (+4 %), spinning waits.
@@ -105,8 +101,7 @@ constexpr uint32_t kRegsCtl = 48;
 constexpr uint32_t kRegsSoftmax = 224;
 static_assert(kRegsCtl * 128 + 2 * kRegsSoftmax * 128 <= kRegsLaunch * kThreads,
               "register split exceeds the launch allocation");
-constexpr float kUnseen = -3.0e38f;     // the reference of a row that has seen no key
-constexpr float kSumLimit = 1.152921504606847e18f;   // 2^60: above it the item runs again
+constexpr float kRescaleLog2 = 8.0f;   // how far a row may outgrow its reference (log2 units)
 
 // Scores 32 c .. 32 c + 31 of a row whose visible keys, relative to the tile, are
 // [lo, hi): the others become -inf (a fully visible chunk is left alone).
@@ -173,13 +168,11 @@ template <int N>
 struct At { static constexpr int value = N; };
 
 // One work item: a (request, pair of query tiles, head), by its block index.
-enum Sweep : int { SWEEP_FIRST = 0, SWEEP_MAX = 1, SWEEP_KNOWN = 2 };
 struct Item {
     int bid;     // < 0: no more items
-    int sweep;   // Sweep: the softmax, the row maxima alone, the softmax with them known
     int head, q0, rs, len, kbase, n0, n1;
 };
-constexpr int kDesc = 9;
+constexpr int kDesc = 8;
 static_assert(sizeof(Item) == kDesc * 4, "descriptor size");
 
 // Heaviest pairs of each request first.
@@ -248,9 +241,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint4* clc_answer = reinterpret_cast<uint4*>(smem + Cfg::kBarOff + 320);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + Cfg::kBarOff + 336);
     int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-    volatile int* redo_any = abort_flag + 1;
-    volatile int* redo = abort_flag + 3;  // [4] items to start again, slot it & 3 (-1: none)
-    volatile int* desc = redo + 4;        // [2][kDesc]
+    volatile int* desc = abort_flag + 3;  // [2][kDesc]
 
     const uint32_t warp = warp_id(), lane = lane_id();
     pdl_launch_dependents();
@@ -275,8 +266,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(loads_out, 1);
         mbar_init(clc_full, 1);
         *abort_flag = 0;
-        *redo_any = 0;
-        for (int k = 0; k < 4; ++k) redo[k] = -1;
         fence_barrier_init();
     }
     // The CTA's own block, as far as it does not depend on an earlier kernel, before the wait
@@ -299,12 +288,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem_base = *tmem_slot;
     const WaitCtx wc{abort_flag, p.status};
 
-    // Every role walks the items to their end, all meet, and where a row sum asked for it
-    // they walk the items to run again.
-    auto meet = [&](int pass) -> bool {
-        __syncthreads();
-        return pass == 0 && *redo_any != 0;
-    };
     // The descriptor of the CTA's it-th item, for the producer and issuer warps; false at
     // the end (or when a role has given up).
     auto next_item = [&](uint32_t it, Item* d) -> bool {
@@ -332,7 +315,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool ok = true;
             int st = 0;
             uint32_t ph = 0;
-            uint32_t it = 0, iq = 0;   // descriptors read, items (the end marks have no Q)
+            uint32_t it = 0;   // items
             // An issuer whose wait gave up releases buffers whose fill it has not seen land:
             // once any role has given up (its flag is set before such a release, and read
             // after the release was seen), nothing is filled again.
@@ -343,47 +326,42 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!ready) gone = mbar_wait_slow(a, parity, wc, site) ? *wc.abort : 1;
                 return __all_sync(0xffffffffu, gone == 0);
             };
-            for (int pass = 0;; ++pass) {
-                Item d;
-                for (; ok && next_item(it, &d); ++it, ++iq) {
-                    const int head = d.head, n_max = max(d.n0, d.n1);
-                    uint64_t* qf = &q_full[iq & 1u];
-                    uint8_t* qt = smem + Cfg::kQOff + (iq & 1u) * 2 * Cfg::kTileBytes;
-                    if (!(ok = may_fill(&q_empty[iq & 1u], ((iq >> 1) & 1u) ^ 1u, 122))) break;
-                    if (elect_one()) {
-                        mbar_expect_tx(qf, 2 * Cfg::kTileBytes);
-                        tma_load_2d(qt, &tmQKV, qf, head * D, d.rs + d.q0);
-                        tma_load_2d(qt + Cfg::kTileBytes, &tmQKV, qf, head * D, d.rs + d.q0 + 128);
-                    }
-                    __syncwarp();
-                    for (int j = 0; j < n_max; ++j) {
-                        if (!(ok = may_fill(&kv_empty[st], ph ^ 1u, 121))) break;
-                        uint8_t* kt = smem + Cfg::kKVOff + st * 2 * Cfg::kTileBytes;
-                        if (elect_one()) {
-                            mbar_expect_tx(&kv_full[st], 2 * Cfg::kTileBytes);
-                            tma_load_2d(kt, &tmQKV, &kv_full[st], p.d_b + head * D, d.rs + d.kbase + j * 128);
-                            tma_load_2d(kt + Cfg::kTileBytes, &tmQKV, &kv_full[st], 2 * p.d_b + head * D,
-                                        d.rs + d.kbase + j * 128);
-                        }
-                        __syncwarp();
-                        if (++st == NS) {
-                            st = 0;
-                            ph ^= 1u;
-                        }
-                    }
-                    if (ok && elect_one()) mbar_arrive(loads_out);
-                    __syncwarp();
+            for (Item d; ok && next_item(it, &d); ++it) {
+                const int head = d.head, n_max = max(d.n0, d.n1);
+                uint64_t* qf = &q_full[it & 1u];
+                uint8_t* qt = smem + Cfg::kQOff + (it & 1u) * 2 * Cfg::kTileBytes;
+                if (!(ok = may_fill(&q_empty[it & 1u], ((it >> 1) & 1u) ^ 1u, 122))) break;
+                if (elect_one()) {
+                    mbar_expect_tx(qf, 2 * Cfg::kTileBytes);
+                    tma_load_2d(qt, &tmQKV, qf, head * D, d.rs + d.q0);
+                    tma_load_2d(qt + Cfg::kTileBytes, &tmQKV, qf, head * D, d.rs + d.q0 + 128);
                 }
-                ++it;   // past the end mark
-                if (!meet(pass)) break;
+                __syncwarp();
+                for (int j = 0; j < n_max; ++j) {
+                    if (!(ok = may_fill(&kv_empty[st], ph ^ 1u, 121))) break;
+                    uint8_t* kt = smem + Cfg::kKVOff + st * 2 * Cfg::kTileBytes;
+                    if (elect_one()) {
+                        mbar_expect_tx(&kv_full[st], 2 * Cfg::kTileBytes);
+                        tma_load_2d(kt, &tmQKV, &kv_full[st], p.d_b + head * D, d.rs + d.kbase + j * 128);
+                        tma_load_2d(kt + Cfg::kTileBytes, &tmQKV, &kv_full[st], 2 * p.d_b + head * D,
+                                    d.rs + d.kbase + j * 128);
+                    }
+                    __syncwarp();
+                    if (++st == NS) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
+                }
+                if (ok && elect_one()) mbar_arrive(loads_out);
+                __syncwarp();
             }
-            // (all roles have met: none gives up after this)
+            __syncthreads();   // all roles meet: none gives up after this
             if (__any_sync(0xffffffffu, *wc.abort != 0)) {
                 // copies may be under way whose reader has given up: the last fill of each
                 // ring slot (those from st on a lap earlier) and of each Q buffer; a wait for
                 // the phase before the first passes
                 for (int s = 0; s < NS; ++s) mbar_wait_landed(&kv_full[s], s < st ? ph : ph ^ 1u);
-                for (uint32_t b = 0; b < 2; ++b) mbar_wait_landed(&q_full[b], (((iq + 1u - b) >> 1) - 1u) & 1u);
+                for (uint32_t b = 0; b < 2; ++b) mbar_wait_landed(&q_full[b], (((it + 1u - b) >> 1) - 1u) & 1u);
             }
         } else if (warp == 1 || warp == 2) {
             // ---------------------------------------------------- MMA issuers
@@ -419,118 +397,105 @@ __global__ void __launch_bounds__(kThreads, 1)
             int sl = 0;           // ring slot of the tile in hand, its phase: every role walks
             uint32_t sp = 0;      // all n_max slots of an item
             uint32_t ns = 0, np = 0, no = 0;   // S tiles read, P tiles multiplied, O tiles started
-            int n, n_max, sweep;
-            uint32_t it = 0, iq = 0;   // descriptors read, items (the end marks have no Q)
-            for (int pass = 0;; ++pass) {
-                for (;; ++it, ++iq) {
-                    {
-                        Item d;
-                        if (!next_item(it, &d)) break;
-                        n = w == 0 ? d.n0 : d.n1;
-                        n_max = max(d.n0, d.n1);
-                        sweep = d.sweep;
+            int n, n_max;
+            uint32_t it = 0;   // items
+            for (;; ++it) {
+                {
+                    Item d;
+                    if (!next_item(it, &d)) break;
+                    n = w == 0 ? d.n0 : d.n1;
+                    n_max = max(d.n0, d.n1);
+                }
+                const uint64_t dq = dq0 + (it & 1u) * ((2 * Cfg::kTileBytes) >> 4);
+                auto issue_s = [&](int slot) {
+                    const uint64_t dk = dk0 + static_cast<uint64_t>(slot) * kStageStep;
+                    if (leader) {
+#pragma unroll
+                        for (int k = 0; k < D / 16; ++k)
+                            mma_bf16_ss(ds, dq + 2 * k, dk + 2 * k, IDESC_S, k != 0 ? 1u : 0u);
+                        mma_commit(&s_full[w]);
                     }
-                    const uint64_t dq = dq0 + (iq & 1u) * ((2 * Cfg::kTileBytes) >> 4);
-                    auto issue_s = [&](int slot) {
-                        const uint64_t dk = dk0 + static_cast<uint64_t>(slot) * kStageStep;
+                    __syncwarp();
+                };
+                wait(&q_full[it & 1u], (it >> 1) & 1u, 221);
+                if (n > 0) {
+                    wait(&kv_full[sl], sp, 222);
+                    issue_s(sl);
+                }
+                for (int j = 0; j < n; ++j) {
+                    const int s1 = sl + 1 == NS ? 0 : sl + 1;
+                    const uint32_t p1 = s1 == 0 ? sp ^ 1u : sp;
+                    // the next tile's operands first, so that S_w,j+1 goes out as soon as
+                    // S_w,j has been read (as it has to be before the next item's first)
+                    if (j + 1 < n) wait(&kv_full[s1], p1, 222);
+                    settle(mbar_test_wait_at<kOffFree>(bar, ns & 1u), bar + kOffFree, ns & 1u, 223);
+                    ++ns;
+                    if (j + 1 < n) {
+                        issue_s(s1);
+                    } else {
+                        if (leader) mma_commit(&q_empty[it & 1u]);
+                        __syncwarp();
+                    }
+                    // the item before has had its O_w read
+                    if (j == 0 && no++ > 0) wait(&o_free[w], (no - 2u) & 1u, 225);
+                    // PV in two halves of 64 keys, each issued as soon as softmax w has
+                    // written it (its V tile arrived with the K tile of S_w,j)
+                    const uint64_t dv = dv0 + static_cast<uint64_t>(sl) * kStageStep;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const bool ready = h == 0 ? mbar_test_wait_at<kOffP0>(bar, np & 1u)
+                                                  : mbar_test_wait_at<kOffP1>(bar, np & 1u);
+                        settle(ready, bar + (h == 0 ? kOffP0 : kOffP1), np & 1u, 224);
                         if (leader) {
 #pragma unroll
-                            for (int k = 0; k < D / 16; ++k)
-                                mma_bf16_ss(ds, dq + 2 * k, dk + 2 * k, IDESC_S, k != 0 ? 1u : 0u);
-                            mma_commit(&s_full[w]);
-                        }
-                        __syncwarp();
-                    };
-                    wait(&q_full[iq & 1u], (iq >> 1) & 1u, 221);
-                    if (n > 0) {
-                        wait(&kv_full[sl], sp, 222);
-                        issue_s(sl);
-                    }
-                    for (int j = 0; j < n; ++j) {
-                        const int s1 = sl + 1 == NS ? 0 : sl + 1;
-                        const uint32_t p1 = s1 == 0 ? sp ^ 1u : sp;
-                        // the next tile's operands first, so that S_w,j+1 goes out as soon as
-                        // S_w,j has been read (as it has to be before the next item's first)
-                        if (j + 1 < n) wait(&kv_full[s1], p1, 222);
-                        settle(mbar_test_wait_at<kOffFree>(bar, ns & 1u), bar + kOffFree, ns & 1u, 223);
-                        ++ns;
-                        if (j + 1 < n) {
-                            issue_s(s1);
-                        } else {
-                            if (leader) mma_commit(&q_empty[iq & 1u]);
-                            __syncwarp();
-                        }
-                        if (sweep != SWEEP_MAX) {
-                            // the item before has had its O_w read
-                            if (j == 0 && no++ > 0) wait(&o_free[w], (no - 2u) & 1u, 225);
-                            // PV in two halves of 64 keys, each issued as soon as softmax w has
-                            // written it (its V tile arrived with the K tile of S_w,j)
-                            const uint64_t dv = dv0 + static_cast<uint64_t>(sl) * kStageStep;
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const bool ready = h == 0 ? mbar_test_wait_at<kOffP0>(bar, np & 1u)
-                                                          : mbar_test_wait_at<kOffP1>(bar, np & 1u);
-                                settle(ready, bar + (h == 0 ? kOffP0 : kOffP1), np & 1u, 224);
-                                if (leader) {
-#pragma unroll
-                                    for (int q = 0; q < 4; ++q) {
-                                        // P from TMEM (16 keys = 8 columns); V: rows = keys (the K
-                                        // dimension), d contiguous (MN-major); 16 keys = two 8-row atoms.
-                                        const int kk = 4 * h + q;
-                                        mma_bf16_ts(dout, pa + kk * 8, dv + kk * ((16 * Cfg::kRowBytes) >> 4),
-                                                    IDESC_PV, (j > 0 || kk != 0) ? 1u : 0u);
-                                    }
-                                    if (h == 1) {
-                                        mma_commit(&pv_done[w]);
-                                        mma_commit(&kv_empty[sl]);
-                                    }
-                                }
-                                __syncwarp();
+                            for (int q = 0; q < 4; ++q) {
+                                // P from TMEM (16 keys = 8 columns); V: rows = keys (the K
+                                // dimension), d contiguous (MN-major); 16 keys = two 8-row atoms.
+                                const int kk = 4 * h + q;
+                                mma_bf16_ts(dout, pa + kk * 8, dv + kk * ((16 * Cfg::kRowBytes) >> 4),
+                                            IDESC_PV, (j > 0 || kk != 0) ? 1u : 0u);
                             }
-                            ++np;
-                        } else {
-                            if (leader) mma_commit(&kv_empty[sl]);
-                            __syncwarp();
+                            if (h == 1) {
+                                mma_commit(&pv_done[w]);
+                                mma_commit(&kv_empty[sl]);
+                            }
                         }
-                        sl = s1;
-                        sp = p1;
-                    }
-                    // the other query tile's key tiles past this one's: released in order,
-                    // so that no wait of this warp is ever two fills of a slot ahead
-                    if (n == 0 && leader) mbar_arrive(&q_empty[iq & 1u]);
-                    __syncwarp();
-                    for (int j = n; j < n_max; ++j) {
-                        wait(&kv_full[sl], sp, 226);
-                        if (leader) mbar_arrive(&kv_empty[sl]);
                         __syncwarp();
-                        if (++sl == NS) {
-                            sl = 0;
-                            sp ^= 1u;
-                        }
+                    }
+                    ++np;
+                    sl = s1;
+                    sp = p1;
+                }
+                // the other query tile's key tiles past this one's: released in order,
+                // so that no wait of this warp is ever two fills of a slot ahead
+                if (n == 0 && leader) mbar_arrive(&q_empty[it & 1u]);
+                __syncwarp();
+                for (int j = n; j < n_max; ++j) {
+                    wait(&kv_full[sl], sp, 226);
+                    if (leader) mbar_arrive(&kv_empty[sl]);
+                    __syncwarp();
+                    if (++sl == NS) {
+                        sl = 0;
+                        sp ^= 1u;
                     }
                 }
-                ++it;
-                if (elect_one()) mma_commit(&drain[w]);
-                __syncwarp();
-                // (an early exit must not leave an MMA that still writes TMEM)
-                if (!mbar_wait_warp(&drain[w], static_cast<uint32_t>(pass), wc, 227))
-                    mbar_wait_landed(&drain[w], static_cast<uint32_t>(pass));
-                if (!meet(pass)) break;
             }
+            if (elect_one()) mma_commit(&drain[w]);
+            __syncwarp();
+            // (an early exit must not leave an MMA that still writes TMEM)
+            if (!mbar_wait_warp(&drain[w], 0, wc, 227)) mbar_wait_landed(&drain[w], 0);
+            __syncthreads();
         } else {
             // ---------------------------------------------------- item scheduler
             // The CTA's first item is its own block; once an item's loads are out, the
             // next one is taken over from a block that has not started yet (cluster
-            // launch control), so that its first tiles load under this item's last
-            // ones.  A row sum past the limit ends the taking over; when the items in
-            // flight are done, those marked run again: row maxima, then the softmax.
+            // launch control), so that its first tiles load under this item's last ones.
             // (one item_empty barrier per slot: a softmax group without a tile runs ahead
             // by one item, never by two)
             uint32_t asked = 0;   // requests made
-            auto publish = [&](uint32_t it, int bid, int sweep) -> bool {
+            auto publish = [&](uint32_t it, int bid) -> bool {
                 Item d{};
                 d.bid = bid;
-                d.sweep = sweep;
                 if (bid >= 0) {
                     locate_item(p, bid, d);
                     count_tiles(p, d);
@@ -552,34 +517,22 @@ __global__ void __launch_bounds__(kThreads, 1)
             do {
                 if (!(ok = mbar_wait_warp(loads_out, it & 1u, wc, 134))) break;
                 ++it;
-                bid = -1;
-                if (!__any_sync(0xffffffffu, *redo_any != 0)) {   // one answer for the warp
-                    if (elect_one()) {
-                        mbar_expect_tx(clc_full, 16);
-                        clc_try_cancel(clc_answer, clc_full);
-                    }
-                    __syncwarp();
-                    if (!(ok = mbar_wait_warp(clc_full, asked & 1u, wc, 135))) {
-                        mbar_wait_landed(clc_full, asked & 1u);   // the answer is a copy, too
-                        break;
-                    }
-                    ++asked;
-                    bid = clc_cancelled_block(clc_answer);
-                    fence_async_smem();   // read before the next answer overwrites it
-                    __syncwarp();
+                if (elect_one()) {
+                    mbar_expect_tx(clc_full, 16);
+                    clc_try_cancel(clc_answer, clc_full);
                 }
-            } while (bid >= 0 && (ok = publish(it, bid, SWEEP_FIRST)));
-            if (ok) ok = publish(it++, -1, SWEEP_FIRST);
-            if (meet(0)) {
-                for (int k = 0; k < 4 && ok; ++k) {
-                    const int again = redo[k];
-                    if (again < 0) continue;
-                    ok = publish(it, again, SWEEP_MAX) && publish(it + 1, again, SWEEP_KNOWN);
-                    it += 2;
+                __syncwarp();
+                if (!(ok = mbar_wait_warp(clc_full, asked & 1u, wc, 135))) {
+                    mbar_wait_landed(clc_full, asked & 1u);   // the answer is a copy, too
+                    break;
                 }
-                if (ok) publish(it, -1, SWEEP_FIRST);
-                meet(1);
-            }
+                ++asked;
+                bid = clc_cancelled_block(clc_answer);
+                fence_async_smem();   // read before the next answer overwrites it
+                __syncwarp();
+            } while (bid >= 0 && (ok = publish(it, bid)));
+            if (ok) publish(it, -1);
+            __syncthreads();
         }
     } else {
         setmaxnreg_inc<kRegsSoftmax>();
@@ -626,33 +579,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                 mask_chunk<3>(s, lo, hi, NEG_INF);
             }
         };
-        auto sweep_max = [&]() {
-            m = NEG_INF;
-            for (int j = 0; j < n; ++j) {
-                float s[128];
-                take_s(s);
-                mask_s(s, j);
-                hand_over(At<kOffFree>{});
-                m = fmaxf(m, row_max(s) * sc);
-            }
-        };
-        // P of one tile (2^(s*sc - m) as bf16 pairs) in two halves of 64 keys, each
+        // P of one tile (2^(s*sc - m_ref) as bf16 pairs) in two halves of 64 keys, each
         // handed over once its store has landed.  P_w is free once PV_w of the tile
         // before has completed: the probe's answer comes in under the second chunk's
         // exponentials.
-        auto put_p = [&](const float (&s)[128]) {
+        auto put_p = [&](const float (&s)[128], float m_ref) {
             uint32_t pk[32];
             float rs[8];
-            exp_chunk<0>(s, sc, m, pk, rs);
+            exp_chunk<0>(s, sc, m_ref, pk, rs);
             const bool pv = mbar_test_wait_at<kOffPV>(bar, (np & 1u) ^ 1u);
-            exp_chunk<1>(s, sc, m, pk + 16, rs);
+            exp_chunk<1>(s, sc, m_ref, pk + 16, rs);
             settle(pv, kOffPV, (np & 1u) ^ 1u, 322);
             ++np;
             tmem_st32u(tp, pk);
             tmem_wait_st();
             hand_over(At<kOffP0>{});
-            exp_chunk<2>(s, sc, m, pk, rs);
-            exp_chunk<3>(s, sc, m, pk + 16, rs);
+            exp_chunk<2>(s, sc, m_ref, pk, rs);
+            exp_chunk<3>(s, sc, m_ref, pk + 16, rs);
             tmem_st32u(tp + 32, pk);
             l += tile_sum(rs);
             tmem_wait_st();
@@ -662,108 +605,102 @@ __global__ void __launch_bounds__(kThreads, 1)
         auto wait_last = [&]() {
             settle(mbar_test_wait_at<kOffPV>(bar, (np & 1u) ^ 1u), kOffPV, (np & 1u) ^ 1u, 324);
         };
-        // P and l of every key tile; `known`: m is the row's maximum already
-        auto sweep = [&](bool known) {
+        // m, P and l of every key tile
+        auto sweep = [&]() {
+            m = NEG_INF;
             l = 0.0f;
-            int fresh = known ? 0 : 1;                 // tiles before this one may find rows without reference
             for (int j = 0; j < n; ++j) {
                 float s[128];
                 take_s(s);
                 mask_s(s, j);
-                if (j < fresh) {
-                    // rows that saw no key before take their reference here; where a row
-                    // sees none yet (block-diagonal mask) m stays at kUnseen and its P is 0
-                    const float mx = row_max(s) * sc;
-                    if (m == kUnseen) m = fmaxf(mx, kUnseen);
-                    if (__any_sync(0xffffffffu, m == kUnseen)) fresh = j + 2;
-                }
                 hand_over(At<kOffFree>{});
-                put_p(s);
+                const float mx = row_max(s) * sc;
+                if (j == 0) {
+                    m = mx;
+                } else if (__any_sync(0xffffffffu, mx > m + kRescaleLog2)) {
+                    const float m_new = fmaxf(m, mx);
+                    const float alpha = (m == m_new) ? 1.0f : ex2(m - m_new);
+                    wait_last();   // O_w is free
+#pragma unroll 1
+                    for (int c = 0; c < D; c += 16) {
+                        float o[16];
+                        tmem_ld16(to + c, o);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) o[i] *= alpha;
+                        tmem_st16(to + c, o);
+                    }
+                    l *= alpha;
+                    m = m_new;
+                }
+                // (a row whose keys start in a later tile has m = -inf: its P is 0)
+                put_p(s, (m == NEG_INF) ? 0.0f : m);
             }
         };
         // (few values live across the key tiles: the softmax threads' registers are full,
         // and the item's descriptor stays in its slot until all of them are done with it)
         uint32_t it = 0;
-        for (int pass = 0;; ++pass) {
-            for (bool more = true; more; ++it) {
-                const volatile Item* d = reinterpret_cast<const volatile Item*>(desc + (it & 1u) * kDesc);
-                more = it == 0 || (mbar_wait_warp(&item_full[it & 1u], (it >> 1) & 1u, wc, 131) && d->bid >= 0);
-                n = 0;
-                if (more) {
-                    // visible keys of this row, relative to the first key tile (a row past
-                    // the request's end is never stored: no mask)
-                    Item o;
-                    o.q0 = d->q0;
-                    o.rs = d->rs;
-                    o.len = d->len;
-                    const int qrow = o.q0 + 128 * w + static_cast<int>(quad * 32 + lane);
-                    const bool in = qrow < o.len;
-                    cend = in ? key_hi(p, o.rs, o.len, qrow) : 1 << 30;
-                    cbeg = in ? key_lo(p, o.rs, qrow) : 0;
-                    if (it == 0) {
-                        count_tiles(p, o);
-                        n = w == 0 ? o.n0 : o.n1;
-                    } else {
-                        o.kbase = d->kbase;
-                        n = w == 0 ? d->n0 : d->n1;
-                    }
-                    cend -= o.kbase;
-                    cbeg -= o.kbase;
+        for (bool more = true; more; ++it) {
+            const volatile Item* d = reinterpret_cast<const volatile Item*>(desc + (it & 1u) * kDesc);
+            more = it == 0 || (mbar_wait_warp(&item_full[it & 1u], (it >> 1) & 1u, wc, 131) && d->bid >= 0);
+            n = 0;
+            if (more) {
+                // visible keys of this row, relative to the first key tile (a row past
+                // the request's end is never stored, but shares its warp's votes: one key)
+                Item o;
+                o.q0 = d->q0;
+                o.rs = d->rs;
+                o.len = d->len;
+                const int qrow = o.q0 + 128 * w + static_cast<int>(quad * 32 + lane);
+                const bool in = qrow < o.len;
+                cend = in ? key_hi(p, o.rs, o.len, qrow) : 1;
+                cbeg = in ? key_lo(p, o.rs, qrow) : 0;
+                if (it == 0) {
+                    count_tiles(p, o);
+                    n = w == 0 ? o.n0 : o.n1;
+                } else {
+                    o.kbase = d->kbase;
+                    n = w == 0 ? d->n0 : d->n1;
                 }
-                if (n > 0 && d->sweep == SWEEP_MAX) {
-                    sweep_max();
-                } else if (n > 0) {
-                    if (d->sweep == SWEEP_FIRST) m = kUnseen;
-                    sweep(d->sweep == SWEEP_KNOWN);
-                    // (what does not need O before the wait for it)
-                    const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane);
-                    const bool valid = qrow < d->len;
-                    const int head = d->head;
-                    const int64_t row = d->rs + qrow;
-                    uint4* d4 = reinterpret_cast<uint4*>(p.out + row * p.d_b + head * D);
-                    const float inv = 1.0f / l;
-                    // the row's log-sum-exp for a backward pass: P = 2^(s sc - (m + log2 l))
-                    if (kLse && valid)
-                        p.lse[static_cast<int64_t>(head) * p.req_start[p.n_req] + row] = m + log2f(l);
-                    wait_last();
-                    // O_w into registers, so that the next item may overwrite it
-                    float o[D];
-                    if constexpr (D == 64) {
-                        tmem_ld64(to, o);
-                    } else {
-                        tmem_ld32(to, o);
-                    }
-                    tmem_wait_ld();
-                    hand_over(At<kOffO>{});
-                    if (valid) {
-#pragma unroll
-                        for (int c = 0; c < D; c += 8)
-                            d4[c / 8] = make_uint4(pack_bf16x2(o[c] * inv, o[c + 1] * inv),
-                                                   pack_bf16x2(o[c + 2] * inv, o[c + 3] * inv),
-                                                   pack_bf16x2(o[c + 4] * inv, o[c + 5] * inv),
-                                                   pack_bf16x2(o[c + 6] * inv, o[c + 7] * inv));
-                    }
-                    // values of up to 2^127 can overflow O while l is below the limit
-                    float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // stays 0 while every o is finite
-#pragma unroll
-                    for (int c = 0; c < D; c += 2) {
-                        const int q = c & 2;
-                        ffma2(z[q], z[q + 1], o[c], o[c + 1], 0.0f, 0.0f, z[q], z[q + 1]);
-                    }
-                    const bool sound = l <= kSumLimit && (z[0] + z[1]) + (z[2] + z[3]) == 0.0f;
-                    if (__any_sync(0xffffffffu, valid && !sound) && d->sweep == SWEEP_FIRST) {
-                        if (lane == 0) {
-                            redo[it & 3u] = d->bid;
-                            *redo_any = 1;
-                        }
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&item_empty[it & 1u]);
+                cend -= o.kbase;
+                cbeg -= o.kbase;
             }
-            tc_fence_before();
-            if (!meet(pass)) break;
+            if (n > 0) {
+                sweep();
+                // (what does not need O before the wait for it)
+                const int qrow = d->q0 + 128 * w + static_cast<int>(quad * 32 + lane);
+                const bool valid = qrow < d->len;
+                const int head = d->head;
+                const int64_t row = d->rs + qrow;
+                uint4* d4 = reinterpret_cast<uint4*>(p.out + row * p.d_b + head * D);
+                const float inv = 1.0f / l;
+                // the row's log-sum-exp for a backward pass: P = 2^(s sc - (m + log2 l))
+                if (kLse && valid)
+                    p.lse[static_cast<int64_t>(head) * p.req_start[p.n_req] + row] = m + log2f(l);
+                wait_last();
+                // O_w into registers, so that the next item may overwrite it
+                float o[D];
+                if constexpr (D == 64) {
+                    tmem_ld64(to, o);
+                } else {
+                    tmem_ld32(to, o);
+                }
+                tmem_wait_ld();
+                hand_over(At<kOffO>{});
+                if (valid) {
+#pragma unroll
+                    for (int c = 0; c < D; c += 8)
+                        d4[c / 8] = make_uint4(pack_bf16x2(o[c] * inv, o[c + 1] * inv),
+                                               pack_bf16x2(o[c + 2] * inv, o[c + 3] * inv),
+                                               pack_bf16x2(o[c + 4] * inv, o[c + 5] * inv),
+                                               pack_bf16x2(o[c + 6] * inv, o[c + 7] * inv));
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&item_empty[it & 1u]);
         }
+        tc_fence_before();
+        __syncthreads();
     }
     if (warp == 1) {
         __syncwarp();

@@ -1,5 +1,5 @@
-"""Attention rows at the limits of their sums: many small weights under a large one, values
-that leave no room above them."""
+"""Attention rows at the limits of their arithmetic: many small weights under a large one, values
+that leave no room above them, one weight that is all of the sum."""
 import numpy as np
 import pytest
 import torch
@@ -64,3 +64,19 @@ def test_huge_values(hd, step):
     bound = 2.0 ** -8 * (mag + np.abs(want)) + 2.0 ** -20 * smax * mag
     assert np.isfinite(got).all()
     assert float((np.abs(got - want) / bound).max()) <= 1.0
+
+
+@pytest.mark.parametrize("key", [5, 200, 699])
+@pytest.mark.parametrize("nh,hd", [(2, 64), (4, 32)])
+def test_one_key_takes_all(nh, hd, key):
+    """One key outweighs all others by 2^46 to 2^57, another factor in each row: the
+    row is that key's value exactly, as its weight is 1, which bf16 holds.  A reference below
+    the row's maximum would round it."""
+    n, db = 700, nh * hd
+    g = torch.Generator("cuda").manual_seed(key)
+    qkv = torch.zeros((n, 3, nh, hd), dtype=torch.bfloat16, device="cuda")
+    qkv[:, 0, :, 0] = 16 + torch.rand((n, nh), generator=g, device="cuda") * 3.5
+    qkv[key, 1, :, 0] = 2.0 * hd ** 0.5
+    qkv[:, 2] = torch.randn((n, nh, hd), generator=g, device="cuda").to(torch.bfloat16)
+    want = qkv[key, 2].reshape(1, db).expand(n, db).clone()
+    assert torch.equal(_call(qkv.reshape(n, 3 * db), db, nh, n), want)

@@ -1265,7 +1265,7 @@ cr_status launch_gemm(const uint16_t* A, int64_t lda, const uint16_t* W, int64_t
     // rounds x (256 + BN) (ties: the wider tile).  The width does not change
     // any output element's K order, so results do not depend on it.
     // The fp32 residual add picks between 160 and 128 that way, and takes 256 instead for
-    // an A that is walked in bands or where that comes out less at rounds x (64 + BN): its
+    // tiles walked in bands or where that comes out less at rounds x (64 + BN): its
     // epilogue, in place on an fp32 tile, grows with BN more than the k-blocks do.  us, 256
     // against the narrower: 95617 tokens at N = 512, 10 rounds instead of 20, the block 1458 /
     // 1590; 9000 x 1024, K = 1024, 2 rounds instead of 4, 19.6 / 22.3; but 3000 x 2048,
@@ -1297,7 +1297,7 @@ cr_status launch_gemm(const uint16_t* A, int64_t lda, const uint16_t* W, int64_t
                 BN = w;
             }
         }
-        if (f32_tile && (static_cast<double>(M) * static_cast<double>(K) * 2.0 > band_from ||
+        if (f32_tile && ((N > 256 && static_cast<double>(M) * static_cast<double>(K) * 2.0 > band_from) ||
                          rounds(256) * (64 + 256) <= rounds(BN) * (64 + BN)))
             BN = 256;
     }

@@ -9,9 +9,10 @@ pytestmark = pytest.mark.gpu
 
 
 # (rows, columns, depth) for 128-wide, 160-wide and 256-wide tiles, and 256-wide ones in
-# bands because the tile updated in place shares L2 with A; ragged rows and columns
+# bands because the tile updated in place shares L2 with A; one column tile, which has no
+# bands, however large A is; ragged rows and columns
 @pytest.mark.parametrize("M,N,K", [(3001, 2048, 512), (5119, 2048, 520), (9001, 1008, 1024), (60001, 528, 512),
-                                   (9001, 4096, 1032)])
+                                   (9001, 4096, 1032), (70001, 128, 512)])
 def test_residual_add_widths(M, N, K):
     g = torch.Generator("cuda").manual_seed(M + N)
     A = torch.randn(M, K, generator=g, device="cuda").to(torch.bfloat16)
